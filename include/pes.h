@@ -58,7 +58,10 @@ typedef struct pes_batch_s* pes_batch_t;
  * digit products of every output coefficient exactly and round the sum once to
  * k limbs (24-bit digits on the FP64 FMA pipe, 28-bit digits with 32x32->64-bit
  * integer multiply-add); results agree to within the last limb's rounding.
- * PES_ARITH_AUTO takes the integer pipe. */
+ * PES_ARITH_AUTO takes the integer pipe, or, for polynomials with many products a
+ * layer at k >= 4 and degrees from 56 to 256 on, integer digits of 18 or 20 bits on the
+ * tensor cores (reported as PES_ARITH_INT).  The choice depends on the sizes of the
+ * monomials, k and d: all plans of one polynomial make the same. */
 enum { PES_ARITH_AUTO = -1, PES_ARITH_FP64 = 0, PES_ARITH_INT = 1 };
 
 typedef struct {
@@ -152,7 +155,8 @@ pes_status pes_plan_complex(const int32_t* supp_ptr, const int32_t* supp_idx, co
  * supp_exp may be NULL) plus its own constant series.  All polynomials share
  * the input series and one job table; the products of every monomial are the
  * ones its own plan would compute, so every output is bit-identical to a plan
- * of that polynomial alone.  Evaluate with pes_eval_system (pes_eval_grad is
+ * of that polynomial alone in the same arithmetic (PES_ARITH_AUTO takes the tensor
+ * cores for a system when it would for each of its polynomials).  Evaluate with pes_eval_system (pes_eval_grad is
  * pes_eval_system with PES_LAYOUT_SERIES); pes_vjp takes one upstream series
  * per polynomial.
  *   P >= 1, poly_ptr: P+1 non-decreasing entries, poly_ptr[0] == 0.
@@ -268,7 +272,9 @@ pes_status pes_get_plan_info(pes_plan_t plan, pes_plan_info* info);
  * arrays.  With pes_partial_grids, an all-reduce (maximum) of the grids,
  * pes_partial_sums, an all-reduce (sum) of the digit sums and pes_round_sums,
  * every rank obtains the value and gradient that one plan of the whole polynomial
- * computes, bit for bit: the addition stage sums the contributions of every
+ * computes, bit for bit, if all of them are given the same arithmetic
+ * (PES_ARITH_INT or PES_ARITH_FP64; PES_ARITH_AUTO goes by the monomials of each plan,
+ * and differs below the last limb's rounding): the addition stage sums the contributions of every
  * output coefficient on the largest grid among them and rounds once, and both
  * the maximum and the sum of integers are exact in any order.  (A sum of the
  * ranks' rounded k-double limbs in floating point would not be.)

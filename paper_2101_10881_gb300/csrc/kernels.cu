@@ -16,18 +16,18 @@
 #include <cstdint>
 #include <map>
 #include <mutex>
-#include <tuple>
 #include <type_traits>
+#include <utility>
 
+#include "dag_sync.cuh"
 #include "digits.cuh"
 #include "kernels.hpp"
 #include "md.cuh"
+#include "slices.cuh"
 
 namespace pes {
 
 namespace {
-
-constexpr int kStatusTimeout = 5;  // PES_ETIMEOUT
 
 __host__ __device__ constexpr size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
@@ -37,22 +37,6 @@ __host__ __device__ constexpr size_t align_up(size_t x, size_t a) { return (x + 
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-
-__device__ __forceinline__ unsigned long long global_timer() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-
-__device__ __forceinline__ int ld_acquire(const int32_t* p) {
-  int v;
-  asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
-
-__device__ __forceinline__ void st_release(int32_t* p, int v) {
-  asm volatile("st.release.gpu.global.b32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
@@ -142,50 +126,6 @@ __device__ __forceinline__ long long acc_value(const Acc64& a) {
   return static_cast<long long>((static_cast<unsigned long long>(static_cast<uint32_t>(a.hi)) << 32) | a.lo);
 }
 __device__ __forceinline__ long long acc_value(double a) { return __double2ll_rn(a); }
-
-__device__ __forceinline__ void set_error(Ctrl* ctrl, int code, long long d0, long long d1) {
-  if (atomicCAS(&ctrl->status, 0, code) == 0) {
-    ctrl->diag[0] = d0;
-    ctrl->diag[1] = d1;
-  }
-  atomicExch(&ctrl->abort, 1);
-}
-
-// Parts of every job of the launch (a split of 0 reads as 1).
-__device__ __forceinline__ int parts(const DagArgs& a) { return a.split > 1 ? a.split : 1; }
-
-// Every part of job `dep` of this call has completed (dep < 0: an input series).
-__device__ __forceinline__ bool is_done(const DagArgs& a, int dep, int epoch) {
-  if (dep < 0) return true;
-  const int s = parts(a);
-  for (int p = 0; p < s; ++p)
-    if (ld_acquire(a.flags + dep * s + p) != epoch) return false;
-  return true;
-}
-
-// Bounded wait until sub-job `f` (a flag index) of this call has completed.
-__device__ bool wait_flag(const DagArgs& a, int f, int epoch, int job) {
-  if (ld_acquire(a.flags + f) == epoch) return true;
-  unsigned long long t0 = global_timer();
-  for (;;) {
-    if (ld_acquire(a.flags + f) == epoch) return true;
-    if (*reinterpret_cast<volatile int32_t*>(&a.ctrl->abort)) return false;
-    if (static_cast<long long>(global_timer() - t0) > a.timeout_ns) {
-      set_error(a.ctrl, kStatusTimeout, f, job);
-      return false;
-    }
-    __nanosleep(200);
-  }
-}
-
-// Bounded wait until every part of job `dep` of this call has completed.
-__device__ bool wait_done(const DagArgs& a, int dep, int epoch, int job) {
-  if (dep < 0) return true;
-  const int s = parts(a);
-  for (int p = 0; p < s; ++p)
-    if (!wait_flag(a, dep * s + p, epoch, job)) return false;
-  return true;
-}
 
 // ---------------------------------------------------------------------------
 // DAG kernel shared-memory layout
@@ -1176,14 +1116,55 @@ __global__ void __launch_bounds__(dag_max_threads(K), INTV ? dag_min_ctas(K) : 1
 // pack / unpack
 // ---------------------------------------------------------------------------
 
+// The workspace rows of one coefficient: digits of B bits, RW words a row.  FP64 and
+// integer arithmetic: int32 digits of 24 or 28 bits, padded to 16 bytes; tensor cores:
+// one word of two slices per digit (slices.cuh).
+template <int K, int AR>
+struct Fmt {
+  static constexpr bool MMA = AR == ARITH_MMA;
+  static constexpr int W = slice_bits(K);
+  static constexpr int B = MMA ? 2 * W : AR == ARITH_INT ? DIGIT_BITS_INT : DIGIT_BITS;
+  static constexpr int L = MMA ? slice_digits(K) : digits_for_k(K, B);
+  static constexpr int RW = MMA ? L : row_words(L, AR == ARITH_INT);
+  // words a sum of series is formed in, digit position 0 the top of its largest grid
+  static constexpr int NW = MMA ? sum_words(K) : L;
+
+  __device__ __forceinline__ static int32_t digit(const int32_t* row, int p) {
+    return MMA ? slice_decode<W>(static_cast<uint32_t>(row[p])) : row[p];
+  }
+  __device__ __forceinline__ static int32_t grid(int32_t word) { return MMA ? meta_grid(word) : word; }
+  // digits D on grid g; gword: where the coefficient's grid is kept
+  template <class T>
+  __device__ __forceinline__ static void store(int32_t* row, int32_t* gword, const T* D, int32_t g) {
+    if constexpr (MMA) {
+      int sq = 0;
+#pragma unroll
+      for (int p = 0; p < L; ++p) {
+        const uint32_t w = slice_encode<W>(static_cast<int32_t>(D[p]));
+        sq += slice_square(w);
+        row[p] = static_cast<int32_t>(w);
+      }
+      *gword = slice_meta(g, sq);
+    } else {
+      *gword = g;
+      int4* dst = reinterpret_cast<int4*>(row);
+#pragma unroll
+      for (int v = 0; v < RW / 4; ++v)
+        dst[v] = make_int4(4 * v < L ? static_cast<int32_t>(D[4 * v]) : 0,
+                           4 * v + 1 < L ? static_cast<int32_t>(D[4 * v + 1]) : 0,
+                           4 * v + 2 < L ? static_cast<int32_t>(D[4 * v + 2]) : 0,
+                           4 * v + 3 < L ? static_cast<int32_t>(D[4 * v + 3]) : 0);
+    }
+  }
+};
+
 // pack: one warp per series; every lane converts coefficients j = lane, lane+32,
 // ... of the caller's k-limb series into L balanced digits on the grid of the
 // leading limb and writes the digit row and grid into the workspace slot.
-template <int K, bool INTV>
+template <int K, int AR>
 __global__ void __launch_bounds__(256) pack_kernel(CopyArgs a) {
-  constexpr int B = INTV ? DIGIT_BITS_INT : DIGIT_BITS;
-  constexpr int L = digits_for_k(K, B);
-  constexpr int RW = row_words(L, INTV);
+  using F = Fmt<K, AR>;
+  constexpr int B = F::B, L = F::L, RW = F::RW;
   const long long row = static_cast<long long>(blockIdx.x) * (blockDim.x / 32) + threadIdx.x / 32;
   const int lane = threadIdx.x & 31;
   if (row >= a.nrows) return;
@@ -1196,24 +1177,16 @@ __global__ void __launch_bounds__(256) pack_kernel(CopyArgs a) {
     int64_t D[L];
     const int32_t g = grid_of<B>(src[j]);
     to_digits<K, L, B>(src + j, r.lstride, g, D);
-    int4* dst = reinterpret_cast<int4*>(rows + static_cast<long long>(j) * RW);
-#pragma unroll
-    for (int v = 0; v < RW / 4; ++v)
-      dst[v] = make_int4(4 * v < L ? static_cast<int32_t>(D[4 * v]) : 0,
-                         4 * v + 1 < L ? static_cast<int32_t>(D[4 * v + 1]) : 0,
-                         4 * v + 2 < L ? static_cast<int32_t>(D[4 * v + 2]) : 0,
-                         4 * v + 3 < L ? static_cast<int32_t>(D[4 * v + 3]) : 0);
-    grids[j] = g;
+    F::store(rows + static_cast<long long>(j) * RW, grids + j, D, g);
   }
 }
 
 // unpack: one warp per series; every lane rounds coefficients of a workspace
 // series (digit form) to k limbs in the caller's buffer.
-template <int K, bool INTV>
+template <int K, int AR>
 __global__ void __launch_bounds__(256) unpack_kernel(CopyArgs a) {
-  constexpr int B = INTV ? DIGIT_BITS_INT : DIGIT_BITS;
-  constexpr int L = digits_for_k(K, B);
-  constexpr int RW = row_words(L, INTV);
+  using F = Fmt<K, AR>;
+  constexpr int B = F::B, L = F::L, RW = F::RW;
   const long long row = static_cast<long long>(blockIdx.x) * (blockDim.x / 32) + threadIdx.x / 32;
   const int lane = threadIdx.x & 31;
   if (row >= a.nrows) return;
@@ -1223,7 +1196,7 @@ __global__ void __launch_bounds__(256) unpack_kernel(CopyArgs a) {
   const int32_t* rows = a.ws + in.ws_base + static_cast<long long>(r.slot) * in.ws_sstride;
   const int32_t* grids = rows + static_cast<long long>(in.S) * RW;
   for (int j = lane; j <= in.d; j += 32) {
-    const int32_t g = grids[j];
+    const int32_t g = F::grid(grids[j]);
     if (g < -100000) {
 #pragma unroll
       for (int l = 0; l < K; ++l) dst[l * r.lstride + j] = 0.0;
@@ -1232,7 +1205,7 @@ __global__ void __launch_bounds__(256) unpack_kernel(CopyArgs a) {
     int64_t E[L + 1];
     E[0] = 0;
 #pragma unroll
-    for (int p = 0; p < L; ++p) E[p + 1] = rows[static_cast<long long>(j) * RW + p];
+    for (int p = 0; p < L; ++p) E[p + 1] = F::digit(rows + static_cast<long long>(j) * RW, p);
     from_digits<K, L, B>(E, g + 1, dst + j, r.lstride);
   }
 }
@@ -1251,16 +1224,15 @@ __global__ void prologue_kernel(Ctrl* ctrl) {
 
 // GROUPED: group_warps warps per output coefficient (block barriers combine
 // them); else one warp per output coefficient and no barrier.
-template <int K, bool INTV, bool GROUPED>
+template <int K, int AR, bool GROUPED>
 __device__ __forceinline__ void add_body(const AddArgs& a, long long items, long long blk) {
-  constexpr int B = INTV ? DIGIT_BITS_INT : DIGIT_BITS;
-  constexpr int L = digits_for_k(K, B);
-  constexpr int RW = row_words(L, INTV);
+  using F = Fmt<K, AR>;
+  constexpr int B = F::B, L = F::L, RW = F::RW, NW = F::NW;
   // a group of group_warps warps per output coefficient (outputs with many
   // contributions spread them over more lanes); every thread reaches the
   // block barriers, so lanes past the last item only skip the work
   __shared__ int32_t gm_s[8];
-  __shared__ long long acc_s[8][L];
+  __shared__ long long acc_s[8][NW];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int gw = GROUPED ? a.group_warps : 1;
   const int G = gw * 32;
@@ -1289,15 +1261,18 @@ __device__ __forceinline__ void add_body(const AddArgs& a, long long items, long
   const long long item =
       (ao.dst_sel == 0 ? 0 : 1 + ao.dst_off / (in.d + 1)) * static_cast<long long>(in.d + 1) + j;
 
-  // common grid: the largest grid of the contributions (mode 2: the one given)
+  // common grid: the largest grid of the contributions (mode 2: the one given;
+  // tensor cores: grids of 28-bit digits are exchanged, and the sum is
+  // formed on the largest grid they stand for)
   int32_t gmax = 2 * GRID_ZERO;
   if (a.mode == 2) {
     gmax = valid ? a.grid_io[item] : gmax;
+    if (F::MMA && gmax >= -100000) gmax = sum_anchor<B>(gmax);
   } else {
     if (valid) {
 #pragma unroll 4
       for (int c = ao.cbeg + gl; c < ao.cend; c += G)
-        gmax = max(gmax, base[static_cast<long long>(a.contrib[c]) * in.ws_sstride + gofs]);
+        gmax = max(gmax, F::grid(base[static_cast<long long>(a.contrib[c]) * in.ws_sstride + gofs]));
     }
 #pragma unroll
     for (int o = 16; o >= 1; o >>= 1) gmax = max(gmax, __shfl_xor_sync(0xffffffffu, gmax, o));
@@ -1307,70 +1282,154 @@ __device__ __forceinline__ void add_body(const AddArgs& a, long long items, long
       for (int t = 0; t < gw; ++t) gmax = max(gmax, gm_s[warp - sw + t]);
     }
     if (a.mode == 1) {
-      if (valid && gl == 0) a.grid_io[item] = gmax;
+      if (valid && gl == 0) a.grid_io[item] = F::MMA && gmax >= -100000 ? sum_grid28<B>(gmax) : gmax;
       return;  // (every thread has passed the group's barrier)
     }
   }
 
-  // every lane sums its contributions' digits, shifted to the common grid
-  int64_t acc[L];
-#pragma unroll
-  for (int p = 0; p < L; ++p) acc[p] = 0;
-  if (valid && gmax >= -100000) {
-#pragma unroll 2
-    for (int c = ao.cbeg + gl; c < ao.cend; c += G) {
-      const int32_t* slot = base + static_cast<long long>(a.contrib[c]) * in.ws_sstride;
-      const int sh = gmax - slot[gofs];  // digits below the common grid's top
-      if (sh >= L) continue;               // below the last digit
-      const int32_t* row = slot + rofs;
-      const long long mu = a.mult ? a.mult[c] : 1;  // the exponent of the variable (Sec. 3)
-#pragma unroll
-      for (int q = 0; q < L; ++q)
-        if (q >= sh) acc[q] += mu * row[q - sh];
+  // tensor cores: the bits below the last 28-bit digit of the sum are
+  // dropped, the f lowest of the digit at position `last` and every digit after it
+  int last = NW - 1, f = 0;
+  int32_t floor28 = 0;
+  if constexpr (F::MMA) {
+    if (gmax >= -100000) {
+      const int32_t G = a.mode == 2 ? a.grid_io[item] : sum_grid28<B>(gmax);
+      floor28 = 28 * (G - digits_for_k(K, DIGIT_BITS_INT));
+      const int32_t e0 = floordiv(floor28, B);
+      f = floor28 - B * e0;
+      last = gmax - 1 - e0;
     }
   }
+
+  // every lane sums its contributions' digits, shifted to the common grid
+  int64_t acc[NW];
+  bool summed = false;
+  if constexpr (F::MMA) {
+    // Few contributions per lane and no factors (the rule is uniform over a group): the
+    // two slices of a word are summed in the halves of one 32-bit word (64 of 2^9 fit),
+    // the last three digits, which may be cut, as digits; the lanes' sums fit 32 bits.
+    // Half the registers and a third of the instructions of the 64-bit sums (the
+    // addition of p2-like, k = 10, took 1.7 times as long with those).
+    if (!a.mult && ao.cend - ao.cbeg <= 32 * G) {
+      summed = true;
+      int32_t half[NW];
 #pragma unroll
-  for (int p = 0; p < L; ++p) {
-    long long v = acc[p];
+      for (int p = 0; p < NW; ++p) half[p] = 0;
+      if (valid && gmax >= -100000) {
+#pragma unroll 2
+        for (int c = ao.cbeg + gl; c < ao.cend; c += G) {
+          const int32_t* slot = base + static_cast<long long>(a.contrib[c]) * in.ws_sstride;
+          const int sh = gmax - F::grid(slot[gofs]);
+          if (sh >= NW) continue;
+          const int32_t* row = slot + rofs - sh;
 #pragma unroll
-    for (int o = 16; o >= 1; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    acc[p] = v;
+          for (int q = 0; q < NW; ++q) {
+            if (q >= sh && q - sh < L) {
+              if (q < NW - 3) {
+                half[q] += slice_halves(static_cast<uint32_t>(row[q]));
+              } else {
+                const int32_t dv = F::digit(row, q);
+                half[q] += q < last ? dv : q == last ? sum_cut(dv, f) : 0;
+              }
+            }
+          }
+        }
+      }
+#pragma unroll
+      for (int p = 0; p < NW; ++p) {
+        int32_t v = half[p];
+        if (p < NW - 3) {
+          const int32_t lo = static_cast<int16_t>(v);
+          v = ((v - lo) >> 16) * (1 << F::W) + lo;
+        }
+        acc[p] = __reduce_add_sync(0xffffffffu, v);
+      }
+    }
+  }
+  if (!summed) {
+#pragma unroll
+    for (int p = 0; p < NW; ++p) acc[p] = 0;
+    if (valid && gmax >= -100000) {
+#pragma unroll 2
+      for (int c = ao.cbeg + gl; c < ao.cend; c += G) {
+        const int32_t* slot = base + static_cast<long long>(a.contrib[c]) * in.ws_sstride;
+        const int sh = gmax - F::grid(slot[gofs]);  // digits below the common grid's top
+        if (sh >= NW) continue;                     // below the last digit
+        const int32_t* row = slot + rofs;
+        const long long mu = a.mult ? a.mult[c] : 1;  // the exponent of the variable (Sec. 3)
+#pragma unroll
+        for (int q = 0; q < NW; ++q) {
+          if (q >= sh && (NW == L || q - sh < L)) {
+            int32_t dv = F::digit(row, q - sh);
+            if (F::MMA && q >= NW - 3) dv = q < last ? dv : q == last ? sum_cut(dv, f) : 0;
+            acc[q] += mu * dv;
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int p = 0; p < NW; ++p) {
+      long long v = acc[p];
+#pragma unroll
+      for (int o = 16; o >= 1; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+      acc[p] = v;
+    }
   }
   if constexpr (GROUPED) {
     if (lane == 0)
 #pragma unroll
-      for (int p = 0; p < L; ++p) acc_s[warp][p] = acc[p];
+      for (int p = 0; p < NW; ++p) acc_s[warp][p] = acc[p];
     __syncthreads();
     if (sw == 0 && lane == 0)
       for (int t = 1; t < gw; ++t)
 #pragma unroll
-        for (int p = 0; p < L; ++p) acc[p] += acc_s[warp + t][p];
+        for (int p = 0; p < NW; ++p) acc[p] += acc_s[warp + t][p];
   }
   if (!valid || gl != 0) return;
   if (a.mode == 2) {
+    if constexpr (F::MMA) {
+      // the same number in 28-bit digits: word w from the bottom weighs 2^(floor28 + 28 w)
+      constexpr int L28 = digits_for_k(K, DIGIT_BITS_INT);
+      long long out[L28];
 #pragma unroll
-    for (int p = 0; p < L; ++p) a.acc_out[item * L + p] = acc[p];
+      for (int p = 0; p < L28; ++p) out[p] = 0;
+      if (gmax >= -100000) {
+        for (int q = 0; q < NW; ++q) {
+          if (q > last) break;
+          const int pos = B * (gmax - 1 - q) - floor28;  // of the word's lowest bit (-f at the last)
+          const long long v = pos < 0 ? acc[q] >> -pos : acc[q];
+          const int b = pos < 0 ? 0 : pos;
+          const int w = b / 28, sft = b % 28;
+          if (w >= L28 - 1) {
+            out[0] += v << (b - 28 * (L28 - 1));
+          } else {
+            const long long hi = v >> (28 - sft);
+            out[L28 - 1 - w] += (v - (hi << (28 - sft))) << sft;
+            out[L28 - 2 - w] += hi;
+          }
+        }
+      }
+      for (int p = 0; p < L28; ++p) a.acc_out[item * L28 + p] = out[p];
+    } else {
+#pragma unroll
+      for (int p = 0; p < L; ++p) a.acc_out[item * L + p] = acc[p];
+    }
     return;
   }
   // acc[p] weighs 2^(B (gmax - 1 - p)): word p + 1 of a sum on grid gmax + 1
-  int64_t E[L + 1];
+  int64_t E[NW + 1];
   E[0] = 0;
 #pragma unroll
-  for (int p = 0; p < L; ++p) E[p + 1] = acc[p];
+  for (int p = 0; p < NW; ++p) E[p + 1] = acc[p];
   if (a.to_ws) {
     int32_t* slot = a.ws + in.ws_base + ao.dst_off * in.ws_sstride;
-    int32_t o[L];
-    const int32_t gz = gmax < -100000 ? GRID_ZERO : sum_to_digits<L, B>(E, gmax + 1, o);
+    int32_t o[NW];  // the first L digits are kept
+    const int32_t gz = gmax < -100000 ? GRID_ZERO : sum_to_digits<NW, B>(E, gmax + 1, o);
     if (gmax < -100000) {
 #pragma unroll
-      for (int p = 0; p < L; ++p) o[p] = 0;
+      for (int p = 0; p < NW; ++p) o[p] = 0;
     }
-    int4* dst = reinterpret_cast<int4*>(slot + rofs);
-#pragma unroll
-    for (int v = 0; v < RW / 4; ++v)
-      dst[v] = make_int4(4 * v < L ? o[4 * v] : 0, 4 * v + 1 < L ? o[4 * v + 1] : 0,
-                         4 * v + 2 < L ? o[4 * v + 2] : 0, 4 * v + 3 < L ? o[4 * v + 3] : 0);
-    slot[gofs] = gz;
+    F::store(slot + rofs, slot + gofs, o, gz);
     return;
   }
   double* dst = a.dst[ao.dst_sel] + ao.dst_off + j * ao.dst_jstride;
@@ -1379,20 +1438,20 @@ __device__ __forceinline__ void add_body(const AddArgs& a, long long items, long
     for (int l = 0; l < K; ++l) dst[l * ao.dst_lstride] = 0.0;
     return;
   }
-  from_digits<K, L, B>(E, gmax + 1, dst, ao.dst_lstride);
+  from_digits<K, NW, B>(E, gmax + 1, dst, ao.dst_lstride);
 }
 
-template <int K, bool INTV>
+template <int K, int AR>
 __global__ void __launch_bounds__(256) add_kernel(AddArgs a, long long items) {
-  add_body<K, INTV, false>(a, items, blockIdx.x);
+  add_body<K, AR, false>(a, items, blockIdx.x);
 }
 
 // Digit sums on their grids (acc[p] weighs 2^(B (g - 1 - p)), g = grids[item])
 // rounded to k limbs, as the addition stage rounds its own sums: item
 // o (d + 1) + j is coefficient j of the value (o = 0) or of d p / d x_{o-1}.
-template <int K, bool INTV>
+template <int K, int AR>
 __host__ __device__ void round_sum_item(const RoundArgs& a, long long item) {
-  constexpr int B = INTV ? DIGIT_BITS_INT : DIGIT_BITS;
+  constexpr int B = AR != ARITH_FP64 ? DIGIT_BITS_INT : DIGIT_BITS;
   constexpr int L = digits_for_k(K, B);
   const long long D1 = a.d + 1;
   const long long o = item / D1, j = item - o * D1;
@@ -1409,33 +1468,33 @@ __host__ __device__ void round_sum_item(const RoundArgs& a, long long item) {
   from_digits<K, L, B>(E, g + 1, dst, ls);
 }
 
-template <int K, bool INTV>
+template <int K, int AR>
 __global__ void __launch_bounds__(256) round_sums_kernel(RoundArgs a, long long items) {
   const long long item = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (item < items) round_sum_item<K, INTV>(a, item);
+  if (item < items) round_sum_item<K, AR>(a, item);
 }
 
-template <int K, bool INTV>
+template <int K, int AR>
 void round_sums_host_k(const RoundArgs& a) {
   const long long items = static_cast<long long>(a.n + 1) * (a.d + 1);
-  for (long long item = 0; item < items; ++item) round_sum_item<K, INTV>(a, item);
+  for (long long item = 0; item < items; ++item) round_sum_item<K, AR>(a, item);
 }
 
-template <int K, bool INTV>
+template <int K, int AR>
 __global__ void __launch_bounds__(256) add_kernel_grouped(AddArgs a, long long items) {
-  add_body<K, INTV, true>(a, items, blockIdx.x);
+  add_body<K, AR, true>(a, items, blockIdx.x);
 }
 
 // Both parts of an addition stage whose outputs are all summed by groups of
 // warps, in one launch: the first nb0 blocks take part 0, the rest part 1 (the
 // branch is uniform over a block, so the group barriers hold).
-template <int K, bool INTV>
+template <int K, int AR>
 __global__ void __launch_bounds__(256) add_kernel_pair(AddArgs a0, long long items0, AddArgs a1, long long items1,
                                                        unsigned nb0) {
   if (blockIdx.x < nb0)
-    add_body<K, INTV, true>(a0, items0, blockIdx.x);
+    add_body<K, AR, true>(a0, items0, blockIdx.x);
   else
-    add_body<K, INTV, true>(a1, items1, blockIdx.x - nb0);
+    add_body<K, AR, true>(a1, items1, blockIdx.x - nb0);
 }
 
 // ---------------------------------------------------------------------------
@@ -1517,7 +1576,8 @@ void* dag_fn(bool tiled, bool narrow) {
   return reinterpret_cast<void*>(&dag_kernel<K, INTV>);
 }
 
-void* dag_kernel_ptr(int k, int arith, bool tiled, bool narrow) {
+void* dag_kernel_ptr(int k, int arith, bool tiled, bool narrow, int dmax) {
+  if (arith == ARITH_MMA) return mma_kernel(k, tiled, dmax);
   const bool iv = arith == ARITH_INT;
   switch (k) {
     case 1: return iv ? dag_fn<1, true>(tiled, narrow) : dag_fn<1, false>(tiled, narrow);
@@ -1535,52 +1595,56 @@ bool narrow_launch(int threads) { return threads > 0 && threads <= kNarrowThread
 
 }  // namespace
 
-int digits_of_k(int k, int arith) { return digits_for_k(k, arith == ARITH_INT ? DIGIT_BITS_INT : DIGIT_BITS); }
+int digits_of_k(int k, int arith) { return digits_for_k(k, arith != ARITH_FP64 ? DIGIT_BITS_INT : DIGIT_BITS); }
 
-int ws_row_words(int k, int arith) { return row_words(digits_of_k(k, arith), arith == ARITH_INT); }
-
-size_t dag_smem_bytes(int k, int arith, int smax, int dmax, int depth, int threads) {
-  return dag_layout(k, digits_of_k(k, arith), arith == ARITH_INT, smax, dmax, depth, threads).total;
+int ws_row_words(int k, int arith) {
+  return arith == ARITH_MMA ? slice_digits(k) : row_words(digits_of_k(k, arith), arith == ARITH_INT);
 }
 
-size_t dag_tiled_smem_bytes(int k, int arith, int tile) {
-  return tile_layout(digits_of_k(k, arith), arith == ARITH_INT, tile).total;
+size_t dag_smem_bytes(int k, int arith, int smax, int dmax, int depth, int threads) {
+  return arith == ARITH_MMA ? mma_smem_bytes(k, dmax, depth)
+                            : dag_layout(k, digits_of_k(k, arith), arith == ARITH_INT, smax, dmax, depth, threads).total;
+}
+
+size_t dag_tiled_smem_bytes(int k, int arith, int tile, int xrows) {
+  return arith == ARITH_MMA ? mma_tiled_smem_bytes(k, tile, xrows)
+                            : tile_layout(digits_of_k(k, arith), arith == ARITH_INT, tile).total;
 }
 
 // The dynamic shared-memory limit is a property of the kernel function on a
 // device, shared by every plan: raise it, never lower it, so that a plan built
 // later for a smaller degree cannot break the launches of an earlier one.
-cudaError_t dag_prepare(int k, int arith, size_t smem, bool tiled) {
-  void* fn = dag_kernel_ptr(k, arith, tiled, false);
-  void* fn_narrow = dag_kernel_ptr(k, arith, tiled, true);  // the same kernel unless k <= 2 whole-series integer
-  if (!fn || !fn_narrow) return cudaErrorInvalidValue;
+cudaError_t dag_prepare(int k, int arith, size_t smem, int dmax, bool tiled) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   static std::mutex mu;
-  static std::map<std::tuple<int, int, int, bool>, size_t> granted;
+  static std::map<std::pair<int, void*>, size_t> granted;
   std::lock_guard<std::mutex> lock(mu);
-  size_t& cur = granted[std::make_tuple(dev, k, arith, tiled)];
-  if (smem <= cur) return cudaSuccess;
-  e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-  if (e == cudaSuccess && fn_narrow != fn)
-    e = cudaFuncSetAttribute(fn_narrow, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-  if (e == cudaSuccess) cur = smem;
-  return e;
+  for (bool narrow : {false, true}) {  // the same kernel unless k <= 2 whole-series integer
+    void* fn = dag_kernel_ptr(k, arith, tiled, narrow, dmax);
+    if (!fn) return cudaErrorInvalidValue;
+    size_t& cur = granted[std::make_pair(dev, fn)];
+    if (smem <= cur) continue;
+    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    if (e != cudaSuccess) return e;
+    cur = smem;
+  }
+  return cudaSuccess;
 }
 
-cudaError_t dag_occupancy(int k, int arith, int threads, size_t smem, int* blocks_per_sm, bool tiled) {
-  void* fn = dag_kernel_ptr(k, arith, tiled, narrow_launch(threads));
+cudaError_t dag_occupancy(int k, int arith, int threads, size_t smem, int dmax, int* blocks_per_sm, bool tiled) {
+  void* fn = dag_kernel_ptr(k, arith, tiled, narrow_launch(threads), dmax);
   if (!fn) return cudaErrorInvalidValue;
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, fn, threads, smem);
 }
 
 cudaError_t launch_dag(const DagArgs& a, int k, int arith, int threads, int grid, cudaStream_t st) {
   const bool tiled = a.tile > 0;
-  void* fn = dag_kernel_ptr(k, arith, tiled, narrow_launch(threads));
+  void* fn = dag_kernel_ptr(k, arith, tiled, narrow_launch(threads), a.dmax);
   if (!fn) return cudaErrorInvalidValue;
-  const size_t smem =
-      tiled ? dag_tiled_smem_bytes(k, arith, a.tile) : dag_smem_bytes(k, arith, a.smax, a.dmax, a.depth, threads);
+  const size_t smem = tiled ? dag_tiled_smem_bytes(k, arith, a.tile, a.xrows)
+                            : dag_smem_bytes(k, arith, a.smax, a.dmax, a.depth, threads);
   DagArgs copy = a;
   void* args[] = {&copy};
   return cudaLaunchKernel(fn, dim3(grid), dim3(threads), args, smem, st);
@@ -1591,27 +1655,28 @@ cudaError_t launch_prologue(Ctrl* ctrl, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-// Launch KERNEL<K, INTV><<<grid, block, 0, st>>>(args...) for run-time k and arith.
-#define PES_DISPATCH_K_ARITH(KERNEL, k, arith, grid, block, st, ...)                        \
-  do {                                                                                      \
-    const bool iv_ = (arith) == ARITH_INT;                                                  \
-    switch (k) {                                                                            \
-      case 1: if (iv_) KERNEL<1, true><<<grid, block, 0, st>>>(__VA_ARGS__);                 \
-              else KERNEL<1, false><<<grid, block, 0, st>>>(__VA_ARGS__); break;             \
-      case 2: if (iv_) KERNEL<2, true><<<grid, block, 0, st>>>(__VA_ARGS__);                 \
-              else KERNEL<2, false><<<grid, block, 0, st>>>(__VA_ARGS__); break;             \
-      case 3: if (iv_) KERNEL<3, true><<<grid, block, 0, st>>>(__VA_ARGS__);                 \
-              else KERNEL<3, false><<<grid, block, 0, st>>>(__VA_ARGS__); break;             \
-      case 4: if (iv_) KERNEL<4, true><<<grid, block, 0, st>>>(__VA_ARGS__);                 \
-              else KERNEL<4, false><<<grid, block, 0, st>>>(__VA_ARGS__); break;             \
-      case 5: if (iv_) KERNEL<5, true><<<grid, block, 0, st>>>(__VA_ARGS__);                 \
-              else KERNEL<5, false><<<grid, block, 0, st>>>(__VA_ARGS__); break;             \
-      case 8: if (iv_) KERNEL<8, true><<<grid, block, 0, st>>>(__VA_ARGS__);                 \
-              else KERNEL<8, false><<<grid, block, 0, st>>>(__VA_ARGS__); break;             \
-      case 10: if (iv_) KERNEL<10, true><<<grid, block, 0, st>>>(__VA_ARGS__);               \
-               else KERNEL<10, false><<<grid, block, 0, st>>>(__VA_ARGS__); break;           \
-      default: return cudaErrorInvalidValue;                                                \
-    }                                                                                       \
+// Launch KERNEL<K, arith><<<grid, block, 0, st>>>(args...) for run-time k and arith.
+#define PES_CASE_ARITH(KERNEL, K, AR, grid, block, st, ...)                       \
+  case 16 * (K) + (AR): KERNEL<K, AR><<<grid, block, 0, st>>>(__VA_ARGS__); break;
+#define PES_CASES_ARITH(KERNEL, AR, grid, block, st, ...)        \
+  PES_CASE_ARITH(KERNEL, 4, AR, grid, block, st, __VA_ARGS__)    \
+  PES_CASE_ARITH(KERNEL, 5, AR, grid, block, st, __VA_ARGS__)    \
+  PES_CASE_ARITH(KERNEL, 8, AR, grid, block, st, __VA_ARGS__)    \
+  PES_CASE_ARITH(KERNEL, 10, AR, grid, block, st, __VA_ARGS__)
+#define PES_CASES_LOW_ARITH(KERNEL, AR, grid, block, st, ...)    \
+  PES_CASE_ARITH(KERNEL, 1, AR, grid, block, st, __VA_ARGS__)    \
+  PES_CASE_ARITH(KERNEL, 2, AR, grid, block, st, __VA_ARGS__)    \
+  PES_CASE_ARITH(KERNEL, 3, AR, grid, block, st, __VA_ARGS__)
+#define PES_DISPATCH_K_ARITH(KERNEL, k, arith, grid, block, st, ...)             \
+  do {                                                                           \
+    switch (16 * (k) + (arith)) {                                                \
+      PES_CASES_LOW_ARITH(KERNEL, 0, grid, block, st, __VA_ARGS__)               \
+      PES_CASES_LOW_ARITH(KERNEL, 1, grid, block, st, __VA_ARGS__)               \
+      PES_CASES_ARITH(KERNEL, 0, grid, block, st, __VA_ARGS__)                   \
+      PES_CASES_ARITH(KERNEL, 1, grid, block, st, __VA_ARGS__)                   \
+      PES_CASES_ARITH(KERNEL, 2, grid, block, st, __VA_ARGS__)                   \
+      default: return cudaErrorInvalidValue;                                     \
+    }                                                                            \
   } while (0)
 
 cudaError_t launch_pack(const CopyArgs& a, int k, int arith, cudaStream_t st) {
@@ -1661,20 +1726,21 @@ cudaError_t launch_round_sums(const RoundArgs& a, int k, int arith, cudaStream_t
   const long long items = static_cast<long long>(a.n + 1) * (a.d + 1);
   if (items == 0) return cudaSuccess;
   const unsigned grid = static_cast<unsigned>((items + 255) / 256);
-  PES_DISPATCH_K_ARITH(round_sums_kernel, k, arith, grid, 256, st, a, items);
+  const int digits = arith == ARITH_FP64 ? ARITH_FP64 : ARITH_INT;  // the sums are in 24- or 28-bit digits
+  PES_DISPATCH_K_ARITH(round_sums_kernel, k, digits, grid, 256, st, a, items);
   return cudaGetLastError();
 }
 
 int round_sums_host(int k, int arith, const RoundArgs& a) {
-  const bool iv = arith == ARITH_INT;
+  const bool iv = arith != ARITH_FP64;
   switch (k) {
-    case 1: iv ? round_sums_host_k<1, true>(a) : round_sums_host_k<1, false>(a); return 0;
-    case 2: iv ? round_sums_host_k<2, true>(a) : round_sums_host_k<2, false>(a); return 0;
-    case 3: iv ? round_sums_host_k<3, true>(a) : round_sums_host_k<3, false>(a); return 0;
-    case 4: iv ? round_sums_host_k<4, true>(a) : round_sums_host_k<4, false>(a); return 0;
-    case 5: iv ? round_sums_host_k<5, true>(a) : round_sums_host_k<5, false>(a); return 0;
-    case 8: iv ? round_sums_host_k<8, true>(a) : round_sums_host_k<8, false>(a); return 0;
-    case 10: iv ? round_sums_host_k<10, true>(a) : round_sums_host_k<10, false>(a); return 0;
+    case 1: iv ? round_sums_host_k<1, ARITH_INT>(a) : round_sums_host_k<1, ARITH_FP64>(a); return 0;
+    case 2: iv ? round_sums_host_k<2, ARITH_INT>(a) : round_sums_host_k<2, ARITH_FP64>(a); return 0;
+    case 3: iv ? round_sums_host_k<3, ARITH_INT>(a) : round_sums_host_k<3, ARITH_FP64>(a); return 0;
+    case 4: iv ? round_sums_host_k<4, ARITH_INT>(a) : round_sums_host_k<4, ARITH_FP64>(a); return 0;
+    case 5: iv ? round_sums_host_k<5, ARITH_INT>(a) : round_sums_host_k<5, ARITH_FP64>(a); return 0;
+    case 8: iv ? round_sums_host_k<8, ARITH_INT>(a) : round_sums_host_k<8, ARITH_FP64>(a); return 0;
+    case 10: iv ? round_sums_host_k<10, ARITH_INT>(a) : round_sums_host_k<10, ARITH_FP64>(a); return 0;
     default: return 1;
   }
 }

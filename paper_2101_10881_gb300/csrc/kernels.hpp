@@ -13,6 +13,7 @@ namespace pes {
 enum : int32_t {
   ARITH_FP64 = 0,  // digit products accumulated with FP64 FMA (exact, flushed every R terms)
   ARITH_INT = 1,   // digit products accumulated with 32x32->64-bit integer multiply-add
+  ARITH_MMA = 2,   // the integer arithmetic on the tensor cores: exact products of 9- or 10-bit slices (slices.cuh)
 };
 
 // Per-plan control block in device memory.
@@ -42,6 +43,7 @@ struct DagArgs {
   long long timeout_ns;     // bound on every wait
   int32_t tile;             // > 0: the tiled kernel, output tiles of `tile` coefficients, `split`
                             // tiles per job (sub-job j * split + t is tile t of job j)
+  int32_t xrows;            // tiled kernel on the tensor cores: coefficients of the first operand staged at once
 };
 
 struct AddArgs {
@@ -107,6 +109,15 @@ __host__ __device__ constexpr int dag_max_regs(int k, bool intv) {
 __host__ __device__ constexpr bool dag_has_narrow(int k, bool intv) { return intv && k <= 2; }
 constexpr int kNarrowThreads = 256;  // widest CTA of the narrow instantiation
 constexpr int kNarrowCtas = 4;       // CTAs per SM its launch bounds declare
+// The most the tensor-core kernels launch with (their accumulators' registers: 168 a
+// thread at k = 8 and 10, 128 at k = 5, 96 at k = 4); a wider request runs with this many.
+__host__ __device__ constexpr int mma_max_threads(int k) { return k >= 8 ? 384 : k >= 5 ? 512 : 640; }
+// The tensor cores take the polynomial of the monomials [m0, m1) (row pointers supp_ptr),
+// degree d, under the automatic arithmetic; `whole`: the integer pipe stages its whole
+// series.  mma_kernels.cu holds the rule's line and its times.
+bool mma_takes(int k, int d, const int32_t* supp_ptr, int32_t m0, int32_t m1, bool whole, size_t optin);
+// Column tiles (8 coefficients) a warp of the tensor-core kernels accumulates at once.
+__host__ __device__ constexpr int mma_group_tiles(int k) { return 3; }
 constexpr int kMaxSplit = 16;  // largest number of parts a convolution job is split into
 
 // Shared-memory footprint of the DAG kernel for (k, arith, smax, dmax) at
@@ -115,7 +126,7 @@ constexpr int kMaxSplit = 16;  // largest number of parts a convolution job is s
 size_t dag_smem_bytes(int k, int arith, int smax, int dmax, int depth, int threads);
 // Shared-memory footprint of the tiled DAG kernel (degrees whose whole series
 // do not fit) for output tiles of `tile` coefficients, any degree.
-size_t dag_tiled_smem_bytes(int k, int arith, int tile);
+size_t dag_tiled_smem_bytes(int k, int arith, int tile, int xrows);
 constexpr int kDefaultTile = 128;  // coefficients per output tile of the tiled kernel
 constexpr int kMaxDegree = 16383;  // largest degree the API accepts
 int digits_of_k(int k, int arith);
@@ -145,6 +156,13 @@ inline int32_t add_group_warps(int64_t max_contrib, int64_t items, int32_t nsm) 
   return gw;
 }
 
+// The tensor-core convolution kernel of k for degrees up to dmax (mma_kernels.cu), its
+// shared memory and its threads per CTA.
+void* mma_kernel(int k, bool tiled, int dmax);
+size_t mma_smem_bytes(int k, int dmax, int depth);
+int mma_threads(int k, int dmax);
+size_t mma_tiled_smem_bytes(int k, int tile, int xrows);
+
 // Launchers (return cudaError_t of the launch).
 cudaError_t launch_prologue(Ctrl* ctrl, cudaStream_t st);
 cudaError_t launch_pack(const CopyArgs& a, int k, int arith, cudaStream_t st);
@@ -158,8 +176,8 @@ cudaError_t launch_add_pair(const AddArgs& a0, int64_t items0, const AddArgs& a1
 cudaError_t launch_round_sums(const RoundArgs& a, int k, int arith, cudaStream_t st);
 // The same rounding on the host (no GPU needed).
 int round_sums_host(int k, int arith, const RoundArgs& a);
-cudaError_t dag_occupancy(int k, int arith, int threads, size_t smem, int* blocks_per_sm, bool tiled = false);
-cudaError_t dag_prepare(int k, int arith, size_t smem, bool tiled = false);
+cudaError_t dag_occupancy(int k, int arith, int threads, size_t smem, int dmax, int* blocks_per_sm, bool tiled = false);
+cudaError_t dag_prepare(int k, int arith, size_t smem, int dmax, bool tiled = false);
 cudaError_t launch_md_binary(int op, int k, const double* x, const double* y, double* out,
                              int64_t count, cudaStream_t st);
 cudaError_t launch_fp64_peak(double* sink, int blocks, int threads, int iters, cudaStream_t st);

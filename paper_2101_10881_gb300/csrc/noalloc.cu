@@ -185,8 +185,9 @@ extern "C" pes_status pes_eval_grad_static(const int32_t* supp_ptr, const int32_
     const int t = std::max((pairs + 31) / 32 * 32, std::min((2 * pairs + 31) / 32 * 32, pes::dag_max_threads(k)));
     if (t <= pes::dag_max_threads(k) &&
         pes::dag_smem_bytes(k, pes::ARITH_INT, S, d, 1, t) <= static_cast<size_t>(optin)) {
-      arith = pes::ARITH_INT;
-      threads = t;
+      arith = pes::mma_takes(k, d, sup.ptr.data(), 0, N, true, static_cast<size_t>(optin)) ? pes::ARITH_MMA
+                                                                                          : pes::ARITH_INT;
+      threads = arith == pes::ARITH_MMA ? pes::mma_threads(k, d) : t;
     }
   }
   const int64_t sstride = pes::ws_slot_words(k, arith, S);
@@ -239,9 +240,9 @@ extern "C" pes_status pes_eval_grad_static(const int32_t* supp_ptr, const int32_
               " does not fit the shared-memory staging of whole series");
     return PES_EUNSUPPORTED_SIZE;
   }
-  STATIC_CUDA(pes::dag_prepare(k, arith, smem));
+  STATIC_CUDA(pes::dag_prepare(k, arith, smem, d));
   int per_sm = 0;
-  STATIC_CUDA(pes::dag_occupancy(k, arith, threads, smem, &per_sm));
+  STATIC_CUDA(pes::dag_occupancy(k, arith, threads, smem, d, &per_sm));
   if (per_sm < 1) {
     set_error("convolution kernel does not fit on an SM");
     return PES_EUNSUPPORTED_SIZE;

@@ -81,20 +81,12 @@ struct CopyTable {
   int32_t n = 0;
 };
 
-// The arithmetic a launch shape uses: PES_ARITH_AUTO takes the integer pipe
-// (whole series in shared memory where they fit, else output tiles).
-int32_t resolve_arith(int32_t k, int32_t requested, int32_t dmax) {
-  (void)k;
-  (void)dmax;
-  return requested != PES_ARITH_AUTO ? requested : pes::ARITH_INT;
-}
-
 // Threads per CTA of the whole-series kernel for the largest degree dmax
 // (`requested` 0: automatic), or 0 when no CTA shape within the cap holds one
 // lane per coefficient pair (integer variant).
 int32_t whole_series_threads(int32_t k, int32_t arith, int32_t dmax, int32_t requested) {
   int32_t t = requested;
-  if (arith == pes::ARITH_INT) {
+  if (arith != pes::ARITH_FP64) {
     // by default two lanes per coefficient pair (one per output coefficient),
     // three at k = 10 (whose CTAs are capped at 256 threads and two per SM:
     // the wider CTA keeps 16 warps per SM where its exchange rows allow two),
@@ -114,8 +106,33 @@ int32_t whole_series_threads(int32_t k, int32_t arith, int32_t dmax, int32_t req
 // depth 1); otherwise the tiled kernel takes it.
 bool whole_series_fits(int32_t k, int32_t arith, int32_t dmax, int32_t requested, int optin) {
   const int32_t t = whole_series_threads(k, arith, dmax, requested);
-  return t > 0 && pes::dag_smem_bytes(k, arith, pes::series_stride(dmax), dmax, 1, t) <= static_cast<size_t>(optin);
+  if (t <= 0) return false;
+  // (tensor cores: of the degrees of the integer pipe's kernel those they can stage too)
+  if (arith == pes::ARITH_MMA && pes::mma_smem_bytes(k, dmax, 1) > static_cast<size_t>(optin)) return false;
+  const int32_t ar = arith == pes::ARITH_MMA ? pes::ARITH_INT : arith;
+  return pes::dag_smem_bytes(k, ar, pes::series_stride(dmax), dmax, 1, t) <= static_cast<size_t>(optin);
 }
+
+// The arithmetic of a plan: PES_ARITH_AUTO takes the integer arithmetic, on the tensor
+// cores where they are faster for every polynomial of it (one, or the P of a system with
+// first monomials poly_ptr).  The rule depends on the monomials' sizes, k and d alone, so
+// that every plan of a polynomial (whole series or tiles, alone, in a batch or without
+// allocations) holds its series in the same form and gives the same bits.
+int32_t resolve_arith(int32_t k, int32_t requested, int32_t d, const pes::Supports& sup,
+                      const std::vector<int32_t>* poly_ptr, int optin) {
+  if (requested != PES_ARITH_AUTO) return requested;
+  const std::vector<int32_t> one{0, sup.N};
+  const std::vector<int32_t>& first = poly_ptr != nullptr ? *poly_ptr : one;
+  const bool whole = whole_series_fits(k, pes::ARITH_INT, d, 0, optin);
+  for (size_t p = 0; p + 1 < first.size(); ++p)
+    if (!pes::mma_takes(k, d, sup.ptr.data(), first[p], first[p + 1], whole, static_cast<size_t>(optin)))
+      return pes::ARITH_INT;
+  return pes::ARITH_MMA;
+}
+
+// Coefficients of the first operand the tiled tensor-core kernel stages at once (with
+// the window of the second they meet).
+constexpr int32_t kStagedRows = 128;
 
 int device_optin() {
   int dev = 0, optin = 0;
@@ -130,8 +147,10 @@ struct Exec {
   int32_t k = 0, arith = 0, threads = 128, ctas_per_sm = 0;
   int32_t smax = 0, dmax = 0;
   int32_t depth = 1, staging = 0;  // staging depth in use; requested (0 = automatic)
+  int32_t threads_req = 0;  // threads per CTA requested (0 = automatic)
   int32_t split = 1, split_req = 0;  // parts per convolution job in use; requested (0 = automatic)
   int32_t tile = 0;  // > 0: the tiled kernel, output tiles of this many coefficients (split = tiles per job)
+  int32_t xrows = 0;  // tiled tensor-core kernel: coefficients of the first operand staged at once
   size_t smem = 0;
   int32_t blocks_per_sm = 0, nsm = 0, optin = 0;
   long long timeout_ns = 0;
@@ -171,7 +190,7 @@ struct Exec {
   // coefficient pairs (measured on the p2-like polynomial at d=152, k=10:
   // within 10 % of the best split for 1 to 128 monomials).
   void choose_split(const std::vector<pes::ConvJob>& jobs) {
-    if (split_req != 0 || arith != pes::ARITH_INT || tile != 0 || jobs.empty()) return;
+    if (split_req != 0 || arith == pes::ARITH_FP64 || tile != 0 || jobs.empty()) return;
     int32_t lo = jobs.front().layer, hi = jobs.front().layer;
     for (const auto& j : jobs) {
       lo = std::min(lo, j.layer);
@@ -179,9 +198,16 @@ struct Exec {
     }
     const double width = static_cast<double>(jobs.size()) / (hi - lo + 1);
     const double ctas = static_cast<double>(blocks_per_sm) * nsm;
-    const int32_t most = std::max(1, (dmax + 2) / 2 / 8);
+    // (tensor cores: one column tile of 8 coefficients)
+    const int32_t most = arith == pes::ARITH_MMA ? (dmax + 8) / 8 : std::max(1, (dmax + 2) / 2 / 8);
+    // Tensor cores: every part stages the whole series, so the parts double only while all
+    // of a layer's run at once, or nearly: 545 jobs a layer on 456 CTAs
+    // took 0.32 / 0.37 ms in one / two parts, 125 0.20 / 0.16 / 0.14 / 0.19 in 1 / 2 / 4 / 8.
     int32_t sp = 1;
-    while (sp < pes::kMaxSplit && 2 * sp <= most && width * sp < ctas) sp *= 2;
+    auto room = [&](int32_t s) {
+      return arith == pes::ARITH_MMA ? 2 * s * width <= 1.1 * ctas : width * s < ctas;
+    };
+    while (sp < pes::kMaxSplit && 2 * sp <= most && room(sp)) sp *= 2;
     split = sp;
   }
 
@@ -189,7 +215,7 @@ struct Exec {
   // when the split is automatic, every split the autotuner may try (1, 2 and
   // half to twice the automatic choice); the tiled kernel flags every tile.
   int32_t flag_parts() const {
-    if (tile > 0 || split_req != 0 || arith != pes::ARITH_INT) return std::max(split, 1);
+    if (tile > 0 || split_req != 0 || arith == pes::ARITH_FP64) return std::max(split, 1);
     return std::max(2, std::min(pes::kMaxSplit, 2 * split));
   }
 
@@ -249,7 +275,7 @@ struct Exec {
   pes_status init(int32_t k_, const pes_options& o, const std::vector<pes::InstInfo>& insts, size_t ws_words_) {
     k = k_;
     arith = o.arith;
-    threads = o.threads;
+    threads = threads_req = o.threads;
     ctas_per_sm = o.ctas_per_sm;
     timeout_ns = (o.timeout_ms > 0 ? o.timeout_ms : 60000) * 1000000LL;
     smax = 8;
@@ -269,7 +295,9 @@ struct Exec {
       // it fits (the autotuner tries both)
       tile = 0;
       threads = whole_series_threads(k, arith, dmax, threads);
-      split = (arith == pes::ARITH_INT && o.split > 0) ? o.split : 1;
+      split = (arith != pes::ARITH_FP64 && o.split > 0) ? o.split : 1;
+      if (arith == pes::ARITH_MMA)
+        threads = o.threads > 0 ? std::min(o.threads, pes::mma_max_threads(k)) : pes::mma_threads(k, dmax);
       depth = (staging == 2 && pes::dag_smem_bytes(k, arith, smax, dmax, 2, threads) <= static_cast<size_t>(optin))
                   ? 2
                   : 1;
@@ -279,7 +307,7 @@ struct Exec {
       // default two per pair (integer variant) or 128 threads (FP64 variant)
       tile = o.tile > 0 ? o.tile : pes::kDefaultTile;
       if (threads == 0)
-        threads = arith == pes::ARITH_INT ? std::min(2 * tile, pes::dag_max_threads(k)) : 128;
+        threads = arith != pes::ARITH_FP64 ? std::min(2 * tile, pes::dag_max_threads(k)) : 128;
       threads = std::max(threads, (tile / 2 + 31) / 32 * 32);
       if (threads > pes::dag_max_threads(k))
         return fail(PES_EUNSUPPORTED_SIZE, "tiles of " + std::to_string(tile) + " coefficients need " +
@@ -287,13 +315,22 @@ struct Exec {
                                                std::to_string(pes::dag_max_threads(k)) + " at k=" + std::to_string(k));
       split = (dmax + tile) / tile;
       depth = 1;
-      smem = pes::dag_tiled_smem_bytes(k, arith, tile);
+      smem = pes::dag_tiled_smem_bytes(k, arith == pes::ARITH_MMA ? pes::ARITH_INT : arith, tile, 0);
+      if (arith == pes::ARITH_MMA && smem <= static_cast<size_t>(optin)) {
+        // (tiles the integer pipe's kernel holds); a warp per group of column tiles
+        // unless asked otherwise
+        threads = std::min(o.threads > 0 ? o.threads
+                                         : 32 * ((tile + 8 * pes::mma_group_tiles(k) - 1) / (8 * pes::mma_group_tiles(k))),
+                           pes::mma_max_threads(k));
+        xrows = std::min(tile, kStagedRows);
+        smem = pes::dag_tiled_smem_bytes(k, arith, tile, xrows);
+      }
     }
     if (smem > static_cast<size_t>(optin))
       return fail(PES_EUNSUPPORTED_SIZE, "degree " + std::to_string(dmax) + " needs " + std::to_string(smem) +
                                              " bytes of shared memory at k=" + std::to_string(k));
-    PES_CUDA(pes::dag_prepare(k, arith, smem, tile > 0));
-    PES_CUDA(pes::dag_occupancy(k, arith, threads, smem, &blocks_per_sm, tile > 0));
+    PES_CUDA(pes::dag_prepare(k, arith, smem, dmax, tile > 0));
+    PES_CUDA(pes::dag_occupancy(k, arith, threads, smem, dmax, &blocks_per_sm, tile > 0));
     if (blocks_per_sm < 1) return fail(PES_EUNSUPPORTED_SIZE, "convolution kernel does not fit on an SM");
     if (ctas_per_sm > 0) blocks_per_sm = std::min(blocks_per_sm, ctas_per_sm);
     pes_status s = upload(&inst, insts);
@@ -314,7 +351,7 @@ struct Exec {
   // shared memory of the convolution kernel at staging depth `dp` with `t`
   // threads per CTA, or 0 if it does not fit
   size_t smem_at(int32_t dp, int32_t t) const {
-    if (tile > 0) return dp == 1 ? pes::dag_tiled_smem_bytes(k, arith, tile) : 0;
+    if (tile > 0) return dp == 1 ? pes::dag_tiled_smem_bytes(k, arith, tile, xrows) : 0;
     const size_t b = pes::dag_smem_bytes(k, arith, smax, dmax, dp, t);
     return b <= static_cast<size_t>(optin) ? b : 0;
   }
@@ -325,16 +362,17 @@ struct Exec {
   pes_status configure(int32_t t, int32_t ctas_cap, int32_t dp, int32_t sp, JobList& L) {
     const size_t b = smem_at(dp, t);
     if (b == 0) return fail(PES_EUNSUPPORTED_SIZE, "staging depth does not fit in shared memory");
-    if (tile > 0 && t < tile / 2) return fail(PES_EUNSUPPORTED_SIZE, "fewer lanes than pairs of a tile");
-    if (tile == 0 && arith == pes::ARITH_INT && L.n > 0 && std::max(1, sp) > L.fparts)
+    if (tile > 0 && arith != pes::ARITH_MMA && t < tile / 2)
+      return fail(PES_EUNSUPPORTED_SIZE, "fewer lanes than pairs of a tile");
+    if (tile == 0 && arith != pes::ARITH_FP64 && L.n > 0 && std::max(1, sp) > L.fparts)
       return fail(PES_EINTERNAL, "parts per job beyond the job flags");
-    PES_CUDA(pes::dag_prepare(k, arith, b, tile > 0));
+    PES_CUDA(pes::dag_prepare(k, arith, b, dmax, tile > 0));
     int bps = 0;
-    PES_CUDA(pes::dag_occupancy(k, arith, t, b, &bps, tile > 0));
+    PES_CUDA(pes::dag_occupancy(k, arith, t, b, dmax, &bps, tile > 0));
     if (bps < 1) return fail(PES_EUNSUPPORTED_SIZE, "configuration does not fit on an SM");
     smem = b;
     depth = dp;
-    if (tile == 0) split = arith == pes::ARITH_INT ? std::max(1, sp) : 1;
+    if (tile == 0) split = arith != pes::ARITH_FP64 ? std::max(1, sp) : 1;
     threads = t;
     blocks_per_sm = ctas_cap > 0 ? std::min(bps, ctas_cap) : bps;
     L.grid = static_cast<int32_t>(std::max<long long>(1, std::min<long long>(
@@ -357,6 +395,7 @@ struct Exec {
     a.split = split;
     a.timeout_ns = timeout_ns;
     a.tile = tile;
+    a.xrows = xrows;
     return a;
   }
 
@@ -574,16 +613,17 @@ pes_status tune_launch(Exec& E, JobList& L, const std::string& key, Run run, cud
   if (!tune_lookup(key, &bt, &bc, &bd, &bs)) {
     const int32_t base = E.threads;
     std::vector<int32_t> ts{base};
-    if (E.arith == pes::ARITH_INT) {
+    if (E.arith != pes::ARITH_FP64) {
+      const int32_t most = E.arith == pes::ARITH_MMA ? pes::mma_max_threads(E.k) : pes::dag_max_threads(E.k);
       for (int32_t t : {base + 32, (base * 3 / 2 + 31) / 32 * 32, base * 2})
-        if (t <= pes::dag_max_threads(E.k) && std::find(ts.begin(), ts.end(), t) == ts.end()) ts.push_back(t);
+        if (t <= most && std::find(ts.begin(), ts.end(), t) == ts.end()) ts.push_back(t);
     } else {
       ts.push_back(256);
     }
     std::vector<int32_t> depths{E.depth};
     if (E.staging == 0) depths = {1, 2};
     std::vector<int32_t> splits{E.split};
-    if (E.split_req == 0 && E.arith == pes::ARITH_INT && E.tile == 0) {
+    if (E.split_req == 0 && E.arith != pes::ARITH_FP64 && E.tile == 0) {
       // the automatic choice (E.split), half and twice it, and 1 and 2
       splits = {1, 2};
       for (int32_t sp : {E.split / 2, E.split, E.split * 2})
@@ -599,9 +639,9 @@ pes_status tune_launch(Exec& E, JobList& L, const std::string& key, Run run, cud
         for (int32_t t : ts) {
           const size_t b = E.smem_at(dp, t);
           if (b == 0) continue;
-          PES_CUDA(pes::dag_prepare(E.k, E.arith, b));
+          PES_CUDA(pes::dag_prepare(E.k, E.arith, b, E.dmax, E.tile > 0));
           int occ = 0;
-          PES_CUDA(pes::dag_occupancy(E.k, E.arith, t, b, &occ));
+          PES_CUDA(pes::dag_occupancy(E.k, E.arith, t, b, E.dmax, &occ, E.tile > 0));
           for (int32_t c = std::max(1, occ); c >= std::max(1, occ - 1); --c) {
             pes_status s = E.configure(t, c, dp, sp, L);
             if (s != PES_OK) continue;
@@ -634,7 +674,7 @@ pes_status tune_launch(Exec& E, JobList& L, const std::string& key, Run run, cud
 
 std::string tune_key(const Exec& E, int64_t njobs, uint64_t signature) {
   char key[200];
-  std::snprintf(key, sizeof(key), "v6_k%d_a%d_t%d_s%d_p%d_T%d_d%d_j%lld_%016llx", E.k, E.arith, E.threads,
+  std::snprintf(key, sizeof(key), "v7_k%d_a%d_t%d_s%d_p%d_T%d_d%d_j%lld_%016llx", E.k, E.arith, E.threads,
                 E.staging, E.split_req, E.tile, E.dmax,
                 static_cast<long long>(njobs), static_cast<unsigned long long>(signature));
   return key;
@@ -746,7 +786,7 @@ pes_status plan_impl(const int32_t* supp_ptr, const int32_t* supp_idx, const int
   const pes::Program1& G = P->prog;
   const int32_t S = pes::series_stride(d);
   const int32_t slots = P->with_vjp ? G.n_slots_vjp : G.n_slots;
-  o.arith = resolve_arith(k, o.arith, d);
+  o.arith = resolve_arith(k, o.arith, d, sup, poly_ptr, device_optin());
   const int64_t sstride = pes::ws_slot_words(k, o.arith, S);
   std::vector<pes::InstInfo> insts{{0, sstride, S, d}};
   s = P->ex.init(k, o, insts, static_cast<size_t>(slots) * static_cast<size_t>(sstride));
@@ -1167,7 +1207,7 @@ extern "C" pes_status pes_get_plan_info(pes_plan_t plan, pes_plan_info* info) {
   info->grid = plan->fwd.grid;
   info->threads = plan->ex.threads;
   info->smem_bytes = static_cast<int32_t>(plan->ex.smem);
-  info->arith = plan->ex.arith;
+  info->arith = plan->ex.arith == pes::ARITH_FP64 ? PES_ARITH_FP64 : PES_ARITH_INT;
   info->staging = plan->ex.depth;
   info->split = plan->ex.split;
   info->complex_series = plan->complex_series ? 1 : 0;
@@ -1279,11 +1319,11 @@ extern "C" pes_status pes_plan_batch_powers(int32_t count, const int32_t* n, con
     B->grad_off[static_cast<size_t>(b) + 1] = B->grad_off[static_cast<size_t>(b)] + k * n[b] * D1;
     prow += N[b] + 1;
     qidx += sup.ptr.back();
-    const int32_t ar = resolve_arith(k, o.arith, d[b]);
+    const int32_t ar = resolve_arith(k, o.arith, d[b], sup, nullptr, optin);
     const bool tiled = o.tile > 0 || !whole_series_fits(k, ar, d[b], o.threads, optin);
     // default CTA: one lane per coefficient within the cap
     const int32_t T = std::min((2 * ((d[b] + 2) / 2) + 31) / 32 * 32, pes::dag_max_threads(k));
-    classes[std::make_tuple(ar, ar == pes::ARITH_INT && !tiled ? T : 0, tiled ? 1 : 0)].push_back(b);
+    classes[std::make_tuple(ar, ar != pes::ARITH_FP64 && !tiled ? T : 0, tiled ? 1 : 0)].push_back(b);
   }
 
   for (auto& cls : classes) {
@@ -1303,7 +1343,7 @@ extern "C" pes_status pes_plan_batch_powers(int32_t count, const int32_t* n, con
     }
     pes_options og = o;
     og.arith = std::get<0>(cls.first);
-    og.threads = std::max(o.threads, std::get<1>(cls.first));
+    og.threads = og.arith == pes::ARITH_MMA ? o.threads : std::max(o.threads, std::get<1>(cls.first));
     if (std::get<2>(cls.first)) og.tile = o.tile > 0 ? o.tile : pes::kDefaultTile;
     s = G->ex.init(k, og, insts, static_cast<size_t>(wsbase));
     if (s != PES_OK) return s;
@@ -1514,7 +1554,7 @@ extern "C" pes_status pes_get_batch_info(pes_batch_t batch, pes_plan_info* info)
   info->grid = static_cast<int32_t>(batch->groups.size());  // number of groups (persistent launches)
   info->threads = E0.threads;
   info->smem_bytes = static_cast<int32_t>(E0.smem);
-  info->arith = E0.arith;
+  info->arith = E0.arith == pes::ARITH_FP64 ? PES_ARITH_FP64 : PES_ARITH_INT;
   info->staging = E0.depth;
   info->split = E0.split;
   for (auto& G : batch->groups) info->tile = std::max(info->tile, G->ex.tile);  // tiled groups, if any
