@@ -1219,47 +1219,68 @@ __global__ void prologue_kernel(Ctrl* ctrl) {
 }
 
 // ---------------------------------------------------------------------------
-// addition stage: warp per output coefficient, exact digit sums, warp shuffles
+// addition stage: warp per output coefficient, exact digit sums, warp shuffles;
+// lane per output coefficient for the rounding
 // ---------------------------------------------------------------------------
 
-// GROUPED: group_warps warps per output coefficient (block barriers combine
-// them); else one warp per output coefficient and no barrier.
+// Tensor cores: the bits below the last 28-bit digit of a sum on grid gmax (G in 28-bit
+// digits) are dropped, the f lowest of the digit at position `last` and every digit after
+// it; its lowest 28-bit word weighs 2^floor28.
+template <int K, int B>
+__device__ __forceinline__ void sum_end(int32_t gmax, int32_t G, int& last, int& f, int32_t& floor28) {
+  floor28 = 28 * (G - digits_for_k(K, DIGIT_BITS_INT));
+  const int32_t e0 = floordiv(floor28, B);
+  f = floor28 - B * e0;
+  last = gmax - 1 - e0;
+}
+
+// The last output whose items start at or before w: 32 starts at a time, one per lane of
+// the warp (w is the warp's).
+__device__ __forceinline__ int find_out(const int64_t* item_ptr, int nouts, long long w) {
+  const int lane = threadIdx.x & 31;
+  int lo = 0, n = nouts;  // the answer lies in [lo, lo + n)
+  while (n > 1) {
+    const int step = (n + 31) / 32;
+    const int at = lo + lane * step;
+    const unsigned below = __ballot_sync(0xffffffffu, at < lo + n && item_ptr[at] <= w);
+    const int b = 31 - __clz(below);  // (lane 0's start is one)
+    n = min(step, n - b * step);
+    lo += b * step;
+  }
+  return lo;
+}
+
+// Item of a real single plan (value: output 0, d p / d x_i: output 1 + i).
+__device__ __forceinline__ long long plan_item(const AddOut& ao, const InstInfo& in, int j) {
+  return (ao.dst_sel == 0 ? 0 : 1 + ao.dst_off / (in.d + 1)) * static_cast<long long>(in.d + 1) + j;
+}
+
+// Item w of a group of gw warps: its sum (digits on grid *grid) and its output *out (mode
+// 1: its grid alone, to a.grid_io).  Every thread reaches the block barriers, so lanes past
+// the last item only skip the work.
 template <int K, int AR, bool GROUPED>
-__device__ __forceinline__ void add_body(const AddArgs& a, long long items, long long blk) {
+__device__ __forceinline__ void add_sums(const AddArgs& a, long long items, long long w, int warp, int lane, int gw,
+                                         int32_t (&gm_s)[8], long long (*acc_s)[Fmt<K, AR>::NW], long long* sum,
+                                         int32_t* grid, int32_t* out) {
   using F = Fmt<K, AR>;
   constexpr int B = F::B, L = F::L, RW = F::RW, NW = F::NW;
-  // a group of group_warps warps per output coefficient (outputs with many
-  // contributions spread them over more lanes); every thread reaches the
-  // block barriers, so lanes past the last item only skip the work
-  __shared__ int32_t gm_s[8];
-  __shared__ long long acc_s[8][NW];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int gw = GROUPED ? a.group_warps : 1;
   const int G = gw * 32;
-  const int sw = warp % gw;                  // warp within the group
-  const int gl = sw * 32 + lane;             // lane within the group
-  const long long w = blk * (8 / gw) + warp / gw;
+  const int sw = warp % gw;       // warp within the group
+  const int gl = sw * 32 + lane;  // lane within the group
   const bool valid = w < items;
   AddOut ao{};
-  int j = 0;
+  int j = 0, o = 0;
   InstInfo in{};
   if (valid) {
-    int lo = 0, hi = a.nouts - 1;
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (a.item_ptr[mid] <= w) lo = mid; else hi = mid - 1;
-    }
-    ao = a.outs[lo];
-    j = static_cast<int>(w - a.item_ptr[lo]);
+    o = find_out(a.item_ptr, a.nouts, w);
+    ao = a.outs[o];
+    j = static_cast<int>(w - a.item_ptr[o]);
     in = a.inst[ao.inst];
   }
   const int32_t* base = a.ws + in.ws_base;
   const long long gofs = static_cast<long long>(in.S) * RW + j;  // grid of coefficient j within a slot
   const long long rofs = static_cast<long long>(j) * RW;         // row of coefficient j within a slot
-
-  // item index of a real single plan (value: output 0, d p / d x_i: output 1 + i)
-  const long long item =
-      (ao.dst_sel == 0 ? 0 : 1 + ao.dst_off / (in.d + 1)) * static_cast<long long>(in.d + 1) + j;
+  const long long item = plan_item(ao, in, j);
 
   // common grid: the largest grid of the contributions (mode 2: the one given;
   // tensor cores: grids of 28-bit digits are exchanged, and the sum is
@@ -1275,7 +1296,7 @@ __device__ __forceinline__ void add_body(const AddArgs& a, long long items, long
         gmax = max(gmax, F::grid(base[static_cast<long long>(a.contrib[c]) * in.ws_sstride + gofs]));
     }
 #pragma unroll
-    for (int o = 16; o >= 1; o >>= 1) gmax = max(gmax, __shfl_xor_sync(0xffffffffu, gmax, o));
+    for (int h = 16; h >= 1; h >>= 1) gmax = max(gmax, __shfl_xor_sync(0xffffffffu, gmax, h));
     if constexpr (GROUPED) {
       if (lane == 0) gm_s[warp] = gmax;
       __syncthreads();
@@ -1283,22 +1304,14 @@ __device__ __forceinline__ void add_body(const AddArgs& a, long long items, long
     }
     if (a.mode == 1) {
       if (valid && gl == 0) a.grid_io[item] = F::MMA && gmax >= -100000 ? sum_grid28<B>(gmax) : gmax;
-      return;  // (every thread has passed the group's barrier)
+      return;
     }
   }
 
-  // tensor cores: the bits below the last 28-bit digit of the sum are
-  // dropped, the f lowest of the digit at position `last` and every digit after it
-  int last = NW - 1, f = 0;
-  int32_t floor28 = 0;
+  int last = NW - 1, f = 0;  // tensor cores: where the sum ends
   if constexpr (F::MMA) {
-    if (gmax >= -100000) {
-      const int32_t G = a.mode == 2 ? a.grid_io[item] : sum_grid28<B>(gmax);
-      floor28 = 28 * (G - digits_for_k(K, DIGIT_BITS_INT));
-      const int32_t e0 = floordiv(floor28, B);
-      f = floor28 - B * e0;
-      last = gmax - 1 - e0;
-    }
+    int32_t floor28 = 0;
+    if (gmax >= -100000) sum_end<K, B>(gmax, a.mode == 2 ? a.grid_io[item] : sum_grid28<B>(gmax), last, f, floor28);
   }
 
   // every lane sums its contributions' digits, shifted to the common grid
@@ -1371,7 +1384,7 @@ __device__ __forceinline__ void add_body(const AddArgs& a, long long items, long
     for (int p = 0; p < NW; ++p) {
       long long v = acc[p];
 #pragma unroll
-      for (int o = 16; o >= 1; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+      for (int h = 16; h >= 1; h >>= 1) v += __shfl_down_sync(0xffffffffu, v, h);
       acc[p] = v;
     }
   }
@@ -1385,8 +1398,25 @@ __device__ __forceinline__ void add_body(const AddArgs& a, long long items, long
 #pragma unroll
         for (int p = 0; p < NW; ++p) acc[p] += acc_s[warp + t][p];
   }
-  if (!valid || gl != 0) return;
+  if (valid && gl == 0) {
+#pragma unroll
+    for (int p = 0; p < NW; ++p) sum[p] = acc[p];
+    *grid = gmax;
+    *out = o;
+  }
+}
+
+// Item w of output o, the sum acc on grid gmax: rounded to k limbs in the caller's buffer,
+// cut to digits in the workspace, or (mode 2) left as digit sums.
+template <int K, int AR>
+__device__ __forceinline__ void add_round(const AddArgs& a, long long w, const long long* acc, int32_t gmax, int o) {
+  using F = Fmt<K, AR>;
+  constexpr int B = F::B, L = F::L, RW = F::RW, NW = F::NW;
+  const AddOut ao = a.outs[o];
+  const InstInfo in = a.inst[ao.inst];
+  const int j = static_cast<int>(w - a.item_ptr[o]);
   if (a.mode == 2) {
+    const long long item = plan_item(ao, in, j);
     if constexpr (F::MMA) {
       // the same number in 28-bit digits: word w from the bottom weighs 2^(floor28 + 28 w)
       constexpr int L28 = digits_for_k(K, DIGIT_BITS_INT);
@@ -1394,6 +1424,9 @@ __device__ __forceinline__ void add_body(const AddArgs& a, long long items, long
 #pragma unroll
       for (int p = 0; p < L28; ++p) out[p] = 0;
       if (gmax >= -100000) {
+        int last, f;
+        int32_t floor28;
+        sum_end<K, B>(gmax, a.grid_io[item], last, f, floor28);
         for (int q = 0; q < NW; ++q) {
           if (q > last) break;
           const int pos = B * (gmax - 1 - q) - floor28;  // of the word's lowest bit (-f at the last)
@@ -1423,13 +1456,13 @@ __device__ __forceinline__ void add_body(const AddArgs& a, long long items, long
   for (int p = 0; p < NW; ++p) E[p + 1] = acc[p];
   if (a.to_ws) {
     int32_t* slot = a.ws + in.ws_base + ao.dst_off * in.ws_sstride;
-    int32_t o[NW];  // the first L digits are kept
-    const int32_t gz = gmax < -100000 ? GRID_ZERO : sum_to_digits<NW, B>(E, gmax + 1, o);
+    int32_t dg[NW];  // the first L digits are kept
+    const int32_t gz = gmax < -100000 ? GRID_ZERO : sum_to_digits<NW, B>(E, gmax + 1, dg);
     if (gmax < -100000) {
 #pragma unroll
-      for (int p = 0; p < NW; ++p) o[p] = 0;
+      for (int p = 0; p < NW; ++p) dg[p] = 0;
     }
-    F::store(slot + rofs, slot + gofs, o, gz);
+    F::store(slot + static_cast<long long>(j) * RW, slot + static_cast<long long>(in.S) * RW + j, dg, gz);
     return;
   }
   double* dst = a.dst[ao.dst_sel] + ao.dst_off + j * ao.dst_jstride;
@@ -1441,6 +1474,36 @@ __device__ __forceinline__ void add_body(const AddArgs& a, long long items, long
   from_digits<K, NW, B>(E, gmax + 1, dst, ao.dst_lstride);
 }
 
+// An output coefficient is summed by a.group_warps warps (GROUPED; block barriers combine
+// them) or one.  A block sums a.rounds times as many as it has groups, one after another,
+// and keeps the sums in shared memory; then it rounds all of them at once, one per lane.
+// Rounding is a serial chain of about 1000 (k = 2) to 9000 (k = 10) instructions that one
+// lane of every group ran while the others idled: it bounded the stage (9945 sums of one or
+// two products, d = 152, k = 10: 80 us, 55 so; eight products of 16 variables, d = 1023,
+// k = 10: 252, 107; 2048 small polynomials, k = 2, whole call: 417, 314).
+template <int K, int AR, bool GROUPED>
+__device__ __forceinline__ void add_body(const AddArgs& a, long long items, long long blk) {
+  using F = Fmt<K, AR>;
+  constexpr int B = F::B, NW = F::NW;
+  // (two sets: a warp may be a round ahead of those that still read)
+  __shared__ int32_t gm_s[2][8];
+  __shared__ long long acc_s[2][8][NW];
+  __shared__ long long sum_s[kAddItems][NW | 1];
+  __shared__ int32_t grid_s[kAddItems], out_s[kAddItems];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int gw = GROUPED ? a.group_warps : 1;
+  const int per = 8 / gw;  // output coefficients of a round
+  const long long first = blk * a.rounds * per;
+  for (int r = 0; r < a.rounds; ++r) {
+    const int at = r * per + warp / gw;
+    add_sums<K, AR, GROUPED>(a, items, first + at, warp, lane, gw, gm_s[r & 1], acc_s[r & 1], sum_s[at],
+                             grid_s + at, out_s + at);
+  }
+  if (a.mode == 1) return;
+  __syncthreads();
+  const int t = threadIdx.x;
+  if (t < a.rounds * per && first + t < items) add_round<K, AR>(a, first + t, sum_s[t], grid_s[t], out_s[t]);
+}
 template <int K, int AR>
 __global__ void __launch_bounds__(256) add_kernel(AddArgs a, long long items) {
   add_body<K, AR, false>(a, items, blockIdx.x);
@@ -1695,17 +1758,26 @@ cudaError_t launch_unpack(const CopyArgs& a, int k, int arith, cudaStream_t st) 
   return cudaGetLastError();
 }
 
+// Rounds of an addition launch's blocks (a.rounds) and its blocks: as many rounds as leave
+// six blocks per SM, at most those whose items a block holds the sums of.
+static unsigned add_blocks(AddArgs& a, int64_t items) {
+  const int64_t per = 8 / a.group_warps;
+  const int64_t sums = (items + per - 1) / per;
+  a.rounds = static_cast<int32_t>(std::max<int64_t>(1, std::min<int64_t>(kAddItems / per, sums / (6 * 152))));
+  return static_cast<unsigned>((sums + a.rounds - 1) / a.rounds);
+}
+
 cudaError_t launch_add(const AddArgs& a, int k, int arith, int64_t items, cudaStream_t st) {
   if (items == 0) return cudaSuccess;
   if (!(a.group_warps == 1 || a.group_warps == 2 || a.group_warps == 4 || a.group_warps == 8))
     return cudaErrorInvalidValue;
   const int warps = 8;
-  const int per_block = warps / a.group_warps;  // output coefficients per block
-  const unsigned grid = static_cast<unsigned>((items + per_block - 1) / per_block);
+  AddArgs b = a;
+  const unsigned grid = add_blocks(b, items);
   if (a.group_warps > 1)
-    PES_DISPATCH_K_ARITH(add_kernel_grouped, k, arith, grid, warps * 32, st, a, static_cast<long long>(items));
+    PES_DISPATCH_K_ARITH(add_kernel_grouped, k, arith, grid, warps * 32, st, b, static_cast<long long>(items));
   else
-    PES_DISPATCH_K_ARITH(add_kernel, k, arith, grid, warps * 32, st, a, static_cast<long long>(items));
+    PES_DISPATCH_K_ARITH(add_kernel, k, arith, grid, warps * 32, st, b, static_cast<long long>(items));
   return cudaGetLastError();
 }
 
@@ -1714,10 +1786,10 @@ cudaError_t launch_add_pair(const AddArgs& a0, int64_t items0, const AddArgs& a1
   const auto grouped = [](int gw) { return gw == 2 || gw == 4 || gw == 8; };
   if (!grouped(a0.group_warps) || !grouped(a1.group_warps)) return cudaErrorInvalidValue;
   const int warps = 8;
-  const long long pb0 = warps / a0.group_warps, pb1 = warps / a1.group_warps;
-  const unsigned nb0 = static_cast<unsigned>((items0 + pb0 - 1) / pb0);
-  const unsigned grid = nb0 + static_cast<unsigned>((items1 + pb1 - 1) / pb1);
-  PES_DISPATCH_K_ARITH(add_kernel_pair, k, arith, grid, warps * 32, st, a0, static_cast<long long>(items0), a1,
+  AddArgs b0 = a0, b1 = a1;
+  const unsigned nb0 = add_blocks(b0, items0);
+  const unsigned grid = nb0 + add_blocks(b1, items1);
+  PES_DISPATCH_K_ARITH(add_kernel_pair, k, arith, grid, warps * 32, st, b0, static_cast<long long>(items0), b1,
                        static_cast<long long>(items1), nb0);
   return cudaGetLastError();
 }

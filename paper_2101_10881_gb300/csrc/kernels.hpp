@@ -46,6 +46,8 @@ struct DagArgs {
   int32_t xrows;            // tiled kernel on the tensor cores: coefficients of the first operand staged at once
 };
 
+constexpr int kAddItems = 32;  // output coefficients whose sums a block of the addition stage holds
+
 struct AddArgs {
   const AddOut* outs;
   int32_t nouts;
@@ -57,6 +59,7 @@ struct AddArgs {
   int32_t* ws;
   double* dst[2];           // k-limb results: caller buffers by selector
   int32_t group_warps;      // warps that share one output coefficient (1, 2, 4 or 8)
+  int32_t rounds;           // items a group sums one after another (set by launch_add)
   // Partial sums of a polynomial split over ranks (real single plans; output o
   // of the value is 0, of d p / d x_i is 1 + i, coefficient j of output o is
   // item o (d + 1) + j):
