@@ -427,7 +427,7 @@ struct Exec {
       a.dst[1] = dst1;
       a.group_warps = A.group_warps[b];
     }
-    if (paired(A)) return pes::launch_add_pair(args[0], A.items[0], args[1], A.items[1], k, arith, st);
+    if (paired(A)) return pes::launch_add_pair(args[1], A.items[1], args[0], A.items[0], k, arith, st);
     for (int b = 0; b < 2; ++b) {
       if (A.items[b] == 0) continue;
       cudaError_t e = pes::launch_add(args[b], k, arith, A.items[b], st);
@@ -436,9 +436,9 @@ struct Exec {
     return cudaSuccess;
   }
 
-  // both parts of an addition stage in one launch (both summed by warp groups)
+  // both parts of an addition stage in one launch
   static bool paired(const AddTable& A) {
-    return A.items[0] > 0 && A.items[1] > 0 && A.group_warps[0] > 1 && A.group_warps[1] > 1;
+    return A.items[0] > 0 && A.items[1] > 0;
   }
 
   // kernels a run_add / run_dag / run_pack / run_unpack call launches
