@@ -1165,15 +1165,19 @@ template <int K, int AR>
 __global__ void __launch_bounds__(256) pack_kernel(CopyArgs a) {
   using F = Fmt<K, AR>;
   constexpr int B = F::B, L = F::L, RW = F::RW;
+  if (a.ctrl != nullptr && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) {
+    a.ctrl->epoch += 1;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) a.ctrl->next[c] = 0;
+  }
   const long long row = static_cast<long long>(blockIdx.x) * (blockDim.x / 32) + threadIdx.x / 32;
-  const int lane = threadIdx.x & 31;
   if (row >= a.nrows) return;
   const CopyRow r = a.rows[row];
   const InstInfo in = a.inst[r.inst];
   const double* src = a.src[r.sel] + r.off;
   int32_t* rows = a.ws + in.ws_base + static_cast<long long>(r.slot) * in.ws_sstride;
   int32_t* grids = rows + static_cast<long long>(in.S) * RW;
-  for (int j = lane; j <= in.d; j += 32) {
+  for (int j = 32 * blockIdx.y + (threadIdx.x & 31); j <= in.d; j += 32 * gridDim.y) {
     int64_t D[L];
     const int32_t g = grid_of<B>(src[j]);
     to_digits<K, L, B>(src + j, r.lstride, g, D);
@@ -1207,14 +1211,6 @@ __global__ void __launch_bounds__(256) unpack_kernel(CopyArgs a) {
 #pragma unroll
     for (int p = 0; p < L; ++p) E[p + 1] = F::digit(rows + static_cast<long long>(j) * RW, p);
     from_digits<K, L, B>(E, g + 1, dst + j, r.lstride);
-  }
-}
-
-__global__ void prologue_kernel(Ctrl* ctrl) {
-  if (threadIdx.x == 0) {
-    ctrl->epoch += 1;
-#pragma unroll
-    for (int c = 0; c < 4; ++c) ctrl->next[c] = 0;
   }
 }
 
@@ -1728,11 +1724,6 @@ cudaError_t launch_dag(const DagArgs& a, int k, int arith, int threads, int grid
   return cudaLaunchKernel(fn, dim3(grid), dim3(threads), args, smem, st);
 }
 
-cudaError_t launch_prologue(Ctrl* ctrl, cudaStream_t st) {
-  prologue_kernel<<<1, 32, 0, st>>>(ctrl);
-  return cudaGetLastError();
-}
-
 // Launch KERNEL<K, arith><<<grid, block, 0, st>>>(args...) for run-time k and arith.
 #define PES_CASE_ARITH(KERNEL, K, AR, grid, block, st, ...)                       \
   case 16 * (K) + (AR): KERNEL<K, AR><<<grid, block, 0, st>>>(__VA_ARGS__); break;
@@ -1758,9 +1749,15 @@ cudaError_t launch_prologue(Ctrl* ctrl, cudaStream_t st) {
   } while (0)
 
 cudaError_t launch_pack(const CopyArgs& a, int k, int arith, cudaStream_t st) {
-  if (a.nrows == 0) return cudaSuccess;
+  if (a.nrows == 0 && a.ctrl == nullptr) return cudaSuccess;
   const int warps = 8;
-  const unsigned grid = static_cast<unsigned>((a.nrows + warps - 1) / warps);
+  const unsigned blocks = static_cast<unsigned>(std::max(1, (a.nrows + warps - 1) / warps));
+  // Few rows: their coefficients, 32 at a time, are dealt to several warps, up to two blocks
+  // per SM.  A digit cut of k = 10 is a serial chain of thousands of instructions, which a
+  // warp went through d / 32 times (66 series, d = 152: 45 -> 17 us; 41 series, d = 1023:
+  // 341 -> 30 us).
+  const unsigned chunks = static_cast<unsigned>(a.dmax / 32 + 1);
+  const dim3 grid(blocks, std::max(1u, std::min(chunks, 304u / blocks)));
   PES_DISPATCH_K_ARITH(pack_kernel, k, arith, grid, warps * 32, st, a);
   return cudaGetLastError();
 }

@@ -18,7 +18,7 @@ enum : int32_t {
 
 // Per-plan control block in device memory.
 struct Ctrl {
-  int32_t epoch;      // incremented once per call by the prologue kernel
+  int32_t epoch;      // incremented once per call by its first pack kernel
   int32_t abort;      // set when any wait gives up
   int32_t status;     // first error code (pes_status), 0 when fine
   int32_t pad0;
@@ -85,6 +85,8 @@ struct RoundArgs {
 struct CopyArgs {
   const CopyRow* rows;
   int32_t nrows;
+  int32_t dmax;          // largest degree of the rows
+  Ctrl* ctrl;            // pack: the call's first launch starts its epoch (else null)
   const InstInfo* inst;
   int32_t* ws;
   const double* src[4];  // pack: caller buffers by selector
@@ -167,7 +169,6 @@ int mma_threads(int k, int dmax);
 size_t mma_tiled_smem_bytes(int k, int tile, int xrows);
 
 // Launchers (return cudaError_t of the launch).
-cudaError_t launch_prologue(Ctrl* ctrl, cudaStream_t st);
 cudaError_t launch_pack(const CopyArgs& a, int k, int arith, cudaStream_t st);
 cudaError_t launch_unpack(const CopyArgs& a, int k, int arith, cudaStream_t st);
 cudaError_t launch_dag(const DagArgs& a, int k, int arith, int threads, int grid, cudaStream_t st);

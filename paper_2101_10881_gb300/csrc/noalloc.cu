@@ -266,6 +266,8 @@ extern "C" pes_status pes_eval_grad_static(const int32_t* supp_ptr, const int32_
   pes::CopyArgs ca{};
   ca.rows = reinterpret_cast<pes::CopyRow*>(base + o_rows);
   ca.nrows = static_cast<int32_t>(rows.size());
+  ca.dmax = d;
+  ca.ctrl = ctrl;
   ca.inst = dinst;
   ca.ws = ws;
   ca.src[0] = coeff;
@@ -299,7 +301,6 @@ extern "C" pes_status pes_eval_grad_static(const int32_t* supp_ptr, const int32_
 
   const int grid = static_cast<int>(std::max<long long>(1, std::min<long long>(static_cast<long long>(per_sm) * nsm,
                                                                                static_cast<long long>(da.njobs))));
-  STATIC_CUDA(pes::launch_prologue(ctrl, st));
   STATIC_CUDA(pes::launch_pack(ca, k, arith, st));
   if (da.njobs > 0) STATIC_CUDA(pes::launch_dag(da, k, arith, threads, grid, st));
   STATIC_CUDA(pes::launch_add(aa, k, arith, item_ptr.back(), st));

@@ -446,11 +446,14 @@ struct Exec {
   static int32_t launches(const JobList& L) { return L.n > 0 ? 1 : 0; }
   static int32_t launches(const CopyTable& C) { return C.n > 0 ? 1 : 0; }
 
-  cudaError_t run_pack(const CopyTable& C, const double* s0, const double* s1, const double* s2,
-                       cudaStream_t st) const {
+  // `first`: the call's first launch, which starts its epoch
+  cudaError_t run_pack(const CopyTable& C, const double* s0, const double* s1, const double* s2, cudaStream_t st,
+                       bool first = true) const {
     pes::CopyArgs a{};
     a.rows = C.rows;
     a.nrows = C.n;
+    a.dmax = dmax;
+    a.ctrl = first ? ctrl : nullptr;
     a.inst = inst;
     a.ws = ws;
     a.src[0] = s0;
@@ -987,7 +990,6 @@ extern "C" pes_status pes_eval_grad(pes_plan_t plan, const double* coeff, const 
   Exec& E = plan->ex;
   {
     auto run = [&](cudaStream_t s2) -> pes_status {
-      PES_CUDA(pes::launch_prologue(E.ctrl, s2));
       PES_CUDA(E.run_pack(plan->pack, coeff, input, nullptr, s2));
       PES_CUDA(E.run_dag(plan->fwd, 0, s2));
       PES_CUDA(E.run_add(plan->add, value, grad, s2));
@@ -997,7 +999,6 @@ extern "C" pes_status pes_eval_grad(pes_plan_t plan, const double* coeff, const 
     if (ts != PES_OK) return ts;
   }
   PES_CUDA(E.mark(0, st));
-  PES_CUDA(pes::launch_prologue(E.ctrl, st));
   PES_CUDA(E.run_pack(plan->pack, coeff, input, nullptr, st));
   PES_CUDA(E.mark(1, st));
   PES_CUDA(E.run_dag(plan->fwd, 0, st));
@@ -1005,7 +1006,7 @@ extern "C" pes_status pes_eval_grad(pes_plan_t plan, const double* coeff, const 
   PES_CUDA(E.run_add(plan->add, value, grad, st));
   PES_CUDA(E.mark(3, st));
   PES_CUDA(E.mark(4, st));
-  E.last_launches = 1 + Exec::launches(plan->pack) + Exec::launches(plan->fwd) + Exec::launches(plan->add);
+  E.last_launches = Exec::launches(plan->pack) + Exec::launches(plan->fwd) + Exec::launches(plan->add);
   return PES_OK;
 }
 
@@ -1054,7 +1055,6 @@ extern "C" pes_status pes_partial_grids(pes_plan_t plan, const double* coeff, co
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   Exec& E = plan->ex;
   auto run = [&](cudaStream_t s2) -> pes_status {
-    PES_CUDA(pes::launch_prologue(E.ctrl, s2));
     PES_CUDA(E.run_pack(plan->pack, coeff, input, nullptr, s2));
     PES_CUDA(E.run_dag(plan->fwd, 0, s2));
     PES_CUDA(E.run_add(plan->add, nullptr, nullptr, s2, 1, grids, nullptr));
@@ -1064,7 +1064,7 @@ extern "C" pes_status pes_partial_grids(pes_plan_t plan, const double* coeff, co
   if (s != PES_OK) return s;
   s = run(st);
   if (s != PES_OK) return s;
-  E.last_launches = 1 + Exec::launches(plan->pack) + Exec::launches(plan->fwd) + Exec::launches(plan->add);
+  E.last_launches = Exec::launches(plan->pack) + Exec::launches(plan->fwd) + Exec::launches(plan->add);
   return PES_OK;
 }
 
@@ -1111,7 +1111,6 @@ extern "C" pes_status pes_eval_system(pes_plan_t plan, const double* coeff, cons
   {
     // both layouts share the job list and its launch shape
     auto run = [&](cudaStream_t s2) -> pes_status {
-      PES_CUDA(pes::launch_prologue(E.ctrl, s2));
       PES_CUDA(E.run_pack(plan->pack, coeff, input, nullptr, s2));
       PES_CUDA(E.run_dag(plan->fwd, 0, s2));
       PES_CUDA(E.run_add(plan->add_mat, value, jac, s2));
@@ -1121,7 +1120,6 @@ extern "C" pes_status pes_eval_system(pes_plan_t plan, const double* coeff, cons
     if (ts != PES_OK) return ts;
   }
   PES_CUDA(E.mark(0, st));
-  PES_CUDA(pes::launch_prologue(E.ctrl, st));
   PES_CUDA(E.run_pack(plan->pack, coeff, input, nullptr, st));
   PES_CUDA(E.mark(1, st));
   PES_CUDA(E.run_dag(plan->fwd, 0, st));
@@ -1129,7 +1127,7 @@ extern "C" pes_status pes_eval_system(pes_plan_t plan, const double* coeff, cons
   PES_CUDA(E.run_add(plan->add_mat, value, jac, st));
   PES_CUDA(E.mark(3, st));
   PES_CUDA(E.mark(4, st));
-  E.last_launches = 1 + Exec::launches(plan->pack) + Exec::launches(plan->fwd) + Exec::launches(plan->add_mat);
+  E.last_launches = Exec::launches(plan->pack) + Exec::launches(plan->fwd) + Exec::launches(plan->add_mat);
   return PES_OK;
 }
 
@@ -1142,18 +1140,17 @@ extern "C" pes_status pes_vjp(pes_plan_t plan, const double* coeff, const double
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   Exec& E = plan->ex;
   PES_CUDA(E.mark(0, st));
-  PES_CUDA(pes::launch_prologue(E.ctrl, st));
   if (reuse_forward) {
     PES_CUDA(E.run_pack(plan->pack_u, nullptr, nullptr, upstream, st));
     PES_CUDA(E.mark(1, st));
     PES_CUDA(E.run_dag(plan->vjp_m, 0, st));
-    E.last_launches = 1 + Exec::launches(plan->pack_u) + Exec::launches(plan->vjp_m);
+    E.last_launches = Exec::launches(plan->pack_u) + Exec::launches(plan->vjp_m);
   } else {
     PES_CUDA(E.run_pack(plan->pack, coeff, input, nullptr, st));
-    PES_CUDA(E.run_pack(plan->pack_u, nullptr, nullptr, upstream, st));
+    PES_CUDA(E.run_pack(plan->pack_u, nullptr, nullptr, upstream, st, false));
     PES_CUDA(E.mark(1, st));
     PES_CUDA(E.run_dag(plan->vjp_fwd, 0, st));
-    E.last_launches = 1 + Exec::launches(plan->pack) + Exec::launches(plan->pack_u) + Exec::launches(plan->vjp_fwd);
+    E.last_launches = Exec::launches(plan->pack) + Exec::launches(plan->pack_u) + Exec::launches(plan->vjp_fwd);
   }
   E.last_launches += Exec::launches(plan->add_g) + Exec::launches(plan->vjp_corr) + Exec::launches(plan->unpack);
   PES_CUDA(E.run_add(plan->add_g, nullptr, nullptr, st));
@@ -1440,7 +1437,6 @@ extern "C" pes_status pes_batch_offsets(pes_batch_t batch, int64_t* coeff_off, i
 static pes_status group_record(Group& G, const double* coeff, const double* input, double* value, double* grad,
                                cudaStream_t st) {
   Exec& E = G.ex;
-  PES_CUDA(pes::launch_prologue(E.ctrl, st));
   PES_CUDA(E.run_pack(G.pack, coeff, input, nullptr, st));
   PES_CUDA(E.run_dag(G.fwd, 0, st));
   PES_CUDA(E.run_add(G.add, value, grad, st));
@@ -1509,7 +1505,7 @@ extern "C" pes_status pes_eval_grad_batch(pes_batch_t batch, const double* coeff
   if (batch->profile) PES_CUDA(cudaEventRecord(batch->ev[1], st));
   batch->last_launches = 0;
   for (auto& G : batch->groups)
-    batch->last_launches += 1 + Exec::launches(G->pack) + Exec::launches(G->fwd) + Exec::launches(G->add);
+    batch->last_launches += Exec::launches(G->pack) + Exec::launches(G->fwd) + Exec::launches(G->add);
   return PES_OK;
 }
 
@@ -1847,7 +1843,7 @@ extern "C" pes_status pes_selftest_timeout(int64_t timeout_ms, int32_t* device_s
     JobList L;
     s = P->ex.make_joblist(L, jobs);
     if (s != PES_OK) return s;
-    PES_CUDA(pes::launch_prologue(P->ex.ctrl, nullptr));
+    PES_CUDA(P->ex.run_pack(CopyTable{}, nullptr, nullptr, nullptr, nullptr));
     PES_CUDA(P->ex.run_dag(L, 0, nullptr));
     st = P->ex.check(nullptr);
     if (st != PES_ETIMEOUT) break;
