@@ -465,16 +465,18 @@ pes_status pes_selftest_timeout(int64_t timeout_ms, int32_t* device_status);
  * Arguments as pes_plan (supports of monomials with exponents one, N, n, d, k)
  * and pes_eval_grad (caller-owned device buffers coeff, input, value, grad;
  * asynchronous on `stream`); the outputs are bit for bit those of pes_plan +
- * pes_eval_grad.  The job tables are compiled on the host at every call and
+ * pes_eval_grad, or, where a plan would take the tensor cores but their longer
+ * series exceed the array, of a plan given PES_ARITH_INT.  The job tables are compiled on the host at every call and
  * copied into the array with cudaMemcpyAsync; nothing calls cudaMalloc,
  * cudaFree or an allocating library routine.  Limits, each rejected with
  * PES_EUNSUPPORTED_SIZE (message in pes_last_error):
  *   - d <= 1023, and the whole operand series of a job must fit one CTA's
  *     shared memory (there is no tiled kernel here): d <= 471 at k=10, 543 at
  *     k=8, 839 at k=5, 991 at k=4;
- *   - tables and workspace within the 64 MiB: at d=152, k=10 a series takes
- *     18,560 bytes of workspace (160 rows of 29 words), so about 3,600 series
- *     fit; the workspace holds 3 n_m - 2 series per monomial of n_m >= 2
+ *   - tables and workspace within the 64 MiB (of the integer pipe's form): at
+ *     d=152, k=10 a series takes 18,560 bytes of workspace (160 rows of 29 words;
+ *     19,200 on the tensor cores), so about 3,600 series fit (3,400, and the
+ *     integer pipe's form from there on); the workspace holds 3 n_m - 2 series per monomial of n_m >= 2
  *     variables, a_0 and the n inputs.
  * Negative d or a NULL buffer is PES_EINVAL, k outside the set
  * PES_EUNSUPPORTED_K.

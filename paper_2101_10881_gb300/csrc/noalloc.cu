@@ -171,29 +171,30 @@ extern "C" pes_status pes_eval_grad_static(const int32_t* supp_ptr, const int32_
   const int32_t S = pes::series_stride(d);
   const int64_t D1 = d + 1;
 
-  // the integer pipe when the whole series of a job fit its staging (one lane
-  // per coefficient pair within the CTA cap, shared memory within the opt-in
-  // limit), else the FP64 pipe
+  // the integer arithmetic when the whole series of a job fit its staging (one
+  // lane per coefficient pair within the CTA cap, shared memory within the opt-in
+  // limit), else the FP64 pipe; on the tensor cores where a plan takes them and
+  // their series, up to 1.54 times as long, fit the array too (below)
   int dev = 0, nsm = 0, optin = 0;
   STATIC_CUDA(cudaGetDevice(&dev));
   STATIC_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
   STATIC_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
   int arith = pes::ARITH_FP64;
   int threads = 128;
+  bool tensor = false;
   {
     const int pairs = (d + 2) / 2;
     const int t = std::max((pairs + 31) / 32 * 32, std::min((2 * pairs + 31) / 32 * 32, pes::dag_max_threads(k)));
     if (t <= pes::dag_max_threads(k) &&
         pes::dag_smem_bytes(k, pes::ARITH_INT, S, d, 1, t) <= static_cast<size_t>(optin)) {
-      arith = pes::mma_takes(k, d, sup.ptr.data(), 0, N, true, static_cast<size_t>(optin)) ? pes::ARITH_MMA
-                                                                                          : pes::ARITH_INT;
-      threads = arith == pes::ARITH_MMA ? pes::mma_threads(k, d) : t;
+      arith = pes::ARITH_INT;
+      threads = t;
+      tensor = pes::mma_takes(k, d, sup.ptr.data(), 0, N, true, static_cast<size_t>(optin));
     }
   }
-  const int64_t sstride = pes::ws_slot_words(k, arith, S);
 
   // tables, in host memory first
-  std::vector<pes::InstInfo> inst{{0, sstride, S, d}};
+  std::vector<pes::InstInfo> inst(1);
   std::vector<pes::CopyRow> rows;
   for (int32_t m = 0; m <= N; ++m) rows.push_back({m * D1, (N + 1) * D1, 0, 0, m, 0});
   for (int32_t i = 0; i < n; ++i) rows.push_back({i * D1, n * D1, 1, 0, 1 + N + i, 0});
@@ -223,7 +224,15 @@ extern "C" pes_status pes_eval_grad_static(const int32_t* supp_ptr, const int32_
   off = align256(off + G.add_src.size() * sizeof(int32_t));
   const size_t table_bytes = off;
   const size_t o_ws = off;
-  const size_t ws_bytes = static_cast<size_t>(G.n_slots) * static_cast<size_t>(sstride) * sizeof(int32_t);
+  const auto ws_size = [&](int ar) {
+    return static_cast<size_t>(G.n_slots) * static_cast<size_t>(pes::ws_slot_words(k, ar, S)) * sizeof(int32_t);
+  };
+  if (tensor && o_ws + ws_size(pes::ARITH_MMA) <= kStaticScratchBytes) {
+    arith = pes::ARITH_MMA;
+    threads = pes::mma_threads(k, d);
+  }
+  inst[0] = pes::InstInfo{0, pes::ws_slot_words(k, arith, S), S, d};
+  const size_t ws_bytes = ws_size(arith);
   if (o_ws + ws_bytes > kStaticScratchBytes) {
     set_error("problem needs " + std::to_string(o_ws + ws_bytes) + " bytes of scratch; the static array holds " +
               std::to_string(kStaticScratchBytes));
