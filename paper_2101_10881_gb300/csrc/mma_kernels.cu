@@ -70,6 +70,7 @@ namespace {
 constexpr int kPairLead = 8;
 constexpr int kPad = 48;               // > 7 + 8 (NT - 1): how far before the series a group's columns run
 constexpr int kZeroGrid = -(1 << 24);  // staged grid (four times the grid) of a zero coefficient
+constexpr int32_t kZeroMeta = -(1 << 30);  // the meta of a zero coefficient
 struct BufLayout {
   int y, x, ga, gb, mx, my, words;  // (mx, my: the metas as copied)
 };
@@ -124,6 +125,7 @@ struct Mma {
 };
 
 constexpr int kMiscWords = 32;
+constexpr int kRangeWord = 8;  // where a Range starts in the misc words
 
 // All of the kernels' shared memory: kMiscWords words, then the buffers.  Staged rows
 // and grids are addressed by byte offsets into it (word indices would cost a shift at
@@ -177,25 +179,84 @@ struct Claim {
 
 // What a warp finds in the staged metas.
 struct Found {
-  int qx, qy;      // largest norms
-  int gmax, gmin;  // largest and smallest grid of a nonzero column coefficient, times four
+  int qx, qy;          // largest norms
+  int gmax, gmin;      // largest and smallest grid of a nonzero column coefficient, times four
+  int x0, x1, y0, y1;  // [x0, x1), [y0, y1): first to last nonzero coefficient of either operand
+  int spread;          // how far apart the grids of two products can lie, times four
 };
 
 // Every warp looks through the metas of the nx Toeplitz and ny column coefficients (that
 // saves a barrier over sharing what it finds); together they leave four times the grids
-// in ga and gb.
+// in ga and gb.  Where the nonzero coefficients lie is looked for when there are zeros, or
+// column coefficients 16 digits apart.
 __device__ __forceinline__ Found split_metas(const int32_t* mx, int32_t* ga, int nx, const int32_t* my, int32_t* gb,
                                              int ny) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
-  Found f{0, 0, -(1 << 30), 1 << 30};
+  Found f{0, 0, -(1 << 30), 1 << 30, 0, nx, 0, ny, 0};
+  bool zeros = false;
   for (int c = lane, u = 0; c < nx; c += 32, ++u) {
     const int32_t w = mx[c];
     if (u % warps == warp) ga[c] = 4 * meta_grid(w);
     f.qx = max(f.qx, w & 255);
+    zeros |= (w & 255) == 0;
   }
   for (int c = lane, u = 0; c < ny; c += 32, ++u) {
     const int32_t w = my[c], g = 4 * meta_grid(w);
     if (u % warps == warp) gb[c] = g;
+    f.qy = max(f.qy, w & 255);
+    f.gmax = max(f.gmax, g > kZeroGrid ? g : f.gmax);
+    f.gmin = min(f.gmin, g > kZeroGrid ? g : f.gmin);
+    zeros |= (w & 255) == 0;
+  }
+  f.qx = __reduce_max_sync(0xffffffffu, f.qx);
+  f.qy = __reduce_max_sync(0xffffffffu, f.qy);
+  f.gmax = __reduce_max_sync(0xffffffffu, f.gmax);
+  f.gmin = __reduce_min_sync(0xffffffffu, f.gmin);
+  if (__any_sync(0xffffffffu, zeros) || f.gmax - f.gmin >= 64) {
+    int x0 = 1 << 20, x1 = 0, y0 = 1 << 20, y1 = 0, xmax = -(1 << 30), xmin = 1 << 30;
+    for (int c = lane; c < nx; c += 32) {
+      const int g = 4 * meta_grid(mx[c]);
+      if (g > kZeroGrid) {
+        x0 = min(x0, c);
+        x1 = c + 1;
+        xmax = max(xmax, g);
+        xmin = min(xmin, g);
+      }
+    }
+    for (int c = lane; c < ny; c += 32)
+      if (4 * meta_grid(my[c]) > kZeroGrid) {
+        y0 = min(y0, c);
+        y1 = c + 1;
+      }
+    f.x0 = __reduce_min_sync(0xffffffffu, x0);
+    f.x1 = __reduce_max_sync(0xffffffffu, x1);
+    f.y0 = __reduce_min_sync(0xffffffffu, y0);
+    f.y1 = __reduce_max_sync(0xffffffffu, y1);
+    xmax = __reduce_max_sync(0xffffffffu, xmax);
+    xmin = __reduce_min_sync(0xffffffffu, xmin);
+    f.spread = f.x1 > 0 && f.y1 > 0 ? xmax - xmin + f.gmax - f.gmin : 0;
+  }
+  return f;
+}
+
+// The same of a chunk in the tiled kernel, whose range tile_range has found.  (Whole warps
+// run through both loops: with those above, the kernel of k = 10 spills and takes 12 %
+// longer.)
+__device__ __forceinline__ Found split_chunk(const int32_t* mx, int32_t* ga, int nx, const int32_t* my, int32_t* gb,
+                                             int ny) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+  Found f{0, 0, -(1 << 30), 1 << 30, 0, nx, 0, ny, 0};
+  for (int c0 = 0, u = 0; c0 < nx; c0 += 32, ++u) {
+    const int c = c0 + lane;
+    const int32_t w = c < nx ? mx[c] : kZeroMeta;
+    if (c < nx && u % warps == warp) ga[c] = 4 * meta_grid(w);
+    f.qx = max(f.qx, w & 255);
+  }
+  for (int c0 = 0, u = 0; c0 < ny; c0 += 32, ++u) {
+    const int c = c0 + lane;
+    const int32_t w = c < ny ? my[c] : kZeroMeta;
+    const int g = 4 * meta_grid(w);
+    if (c < ny && u % warps == warp) gb[c] = g;
     f.qy = max(f.qy, w & 255);
     f.gmax = max(f.gmax, g > kZeroGrid ? g : f.gmax);
     f.gmin = min(f.gmin, g > kZeroGrid ? g : f.gmin);
@@ -205,6 +266,52 @@ __device__ __forceinline__ Found split_metas(const int32_t* mx, int32_t* ga, int
   f.gmax = __reduce_max_sync(0xffffffffu, f.gmax);
   f.gmin = __reduce_min_sync(0xffffffffu, f.gmin);
   return f;
+}
+
+// Where the nonzero coefficients of the two operands lie: [x0, x1) and [y0, y1); far:
+// products can lie L digits below the largest of their column.
+struct Range {
+  int x0, x1, y0, y1, far;
+};
+
+// The terms [begin, end) that meet nonzero coefficients in the columns jlo to jhi.
+__device__ __forceinline__ void nonzero_terms(const volatile Range* r, int jlo, int jhi, int& begin, int& end) {
+  begin = max(r->x0, jlo - r->y1 + 1);
+  end = min(r->x1, jhi - r->y0 + 1);
+}
+
+// The terms [x0, x1) that meet nonzero coefficients in the columns [c0, terms) of an
+// output tile (into the Range of the misc words), by the whole CTA.  (Not inlined: the
+// kernel around it has no register to spare.)
+__device__ __noinline__ void tile_range(const int32_t* gx, const int32_t* gy, int step, int terms, int c0) {
+  Range* r = reinterpret_cast<Range*>(sm + kRangeWord);
+  if (threadIdx.x == 0) *r = Range{terms, 0, terms, 0, 0};
+  __syncthreads();
+  int x0 = terms, x1 = 0, y0 = terms, y1 = 0;
+  for (int i = threadIdx.x; i < terms; i += blockDim.x) {
+    const bool nx = 4 * meta_grid(__ldcg(gx + i)) > kZeroGrid, ny = 4 * meta_grid(__ldcg(gy + i * step)) > kZeroGrid;
+    x0 = nx ? min(x0, i) : x0;
+    x1 = nx ? i + 1 : x1;
+    y0 = ny ? min(y0, i) : y0;
+    y1 = ny ? i + 1 : y1;
+  }
+  x0 = __reduce_min_sync(0xffffffffu, x0);
+  x1 = __reduce_max_sync(0xffffffffu, x1);
+  y0 = __reduce_min_sync(0xffffffffu, y0);
+  y1 = __reduce_max_sync(0xffffffffu, y1);
+  if ((threadIdx.x & 31) == 0) {
+    atomicMin(&r->x0, x0);
+    atomicMax(&r->x1, x1);
+    atomicMin(&r->y0, y0);
+    atomicMax(&r->y1, y1);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const int begin = max(r->x0, c0 - r->y1 + 1), end = min(r->x1, terms - r->y0);
+    r->x0 = begin;
+    r->x1 = end;
+  }
+  __syncthreads();
 }
 
 // The columns' grids lie close enough for their rows to be shifted to the largest.
@@ -292,6 +399,23 @@ struct Terms {
   bool flat;  // columns staged on one grid, gmax
   int gmax;
 };
+
+// From the first to the last of the terms [begin, end) whose product reaches a column: its
+// grid lies above the column's `least` (three tiles; four times the grids at ga, and, of
+// the lane's columns, at gb).
+__device__ __forceinline__ int2 reaching_terms(int ga, int gb, int begin, int end, int3 least) {
+  int first = end, last = begin;
+#pragma unroll 2
+  for (int i = begin + static_cast<int>(threadIdx.x & 3); i < end; i += 4) {
+    const int gx = static_cast<int>(lds(ga + 4 * i)), at = gb - 4 * i;
+    const int y0 = static_cast<int>(lds(at)), y1 = static_cast<int>(lds(at - 32)), y2 = static_cast<int>(lds(at - 64));
+    if (gx + y0 > least.x || gx + y1 > least.y || gx + y2 > least.z) {
+      first = min(first, i);
+      last = i + 1;
+    }
+  }
+  return make_int2(__reduce_min_sync(0xffffffffu, first), __reduce_max_sync(0xffffffffu, last));
+}
 
 // A group of up to NT column tiles of one warp: tile t holds the columns 8 t before those
 // of tile 0.
@@ -678,9 +802,14 @@ __device__ __forceinline__ void add_rows(const int32_t* xs, const int32_t* ys, i
 
 // The nt tiles from the o-th longest on of a job whose series are staged, by one warp:
 // tile o holds the columns d - 7 - 8 o to d - 8 o, so that the ragged tile is the one
-// with fewest terms.  With `shares` > 1 (nt = 1), this warp adds the terms of share
-// `share` of the tile only, the shares meet in `scratch` and the first warp of the tile
-// stores them; the whole CTA calls together then (nt = 0: nothing to add).
+// with fewest terms.  Terms at either end that reach no column (zero coefficients, or
+// products L digits below the largest of every column) are left out, as the integer pipe
+// leaves out every such term.  All pairs of 128 variables, d = 152, k = 4 (integer pipe;
+// all terms; here): coefficients of degree 0 1.87; 2.40; 1.56 ms, inputs of degree 1 1.34;
+// 2.41; 1.27 ms, exponential inputs 2.01; 2.36; 1.62 ms.  The range of the nonzero
+// coefficients is read from shared memory for every group: registers are what the term
+// loop has fewest of.  (128 products of 64, k = 10, uniform series: 6.13 ms without the
+// ranges, 6.20 with them.)
 template <int K, bool PAIRS>
 __device__ __forceinline__ void columns(int d, int o, int nt, Terms a, bool rev, int32_t* zrows, int32_t* zmeta) {
   constexpr int SW = Mma<K>::SW, NT = Mma<K>::NT, NB = Mma<K>::NB;
@@ -711,6 +840,24 @@ __device__ __forceinline__ void columns(int d, int o, int nt, Terms a, bool rev,
     if (t >= nt) gm[t] = 2 * kZeroGrid;
   }
   grp.set_grids(gm);
+  const volatile Range* range = reinterpret_cast<const volatile Range*>(sm + kRangeWord);
+  int begin, end;
+  nonzero_terms(range, max(0, j0 - 8 * (nt - 1)), j0 + 7, begin, end);
+  if (range->far != 0 && begin < min(end, n[0])) {
+    static_assert(NT == 3, "reaching_terms takes three tiles");
+    const int reach = 4 * Mma<K>::L;
+    const int2 r = reaching_terms(a.ga, a.gb, begin, min(end, n[0]),
+                                  make_int3(grp.gs[0] - reach, nt > 1 ? grp.gs[1] - reach : 1 << 30,
+                                            nt > 2 ? grp.gs[2] - reach : 1 << 30));
+    begin = r.x;
+    end = r.y;
+  }
+#pragma unroll
+  for (int t = 0; t < NT; ++t) n[t] = min(n[t], end) - begin;
+  a.x += begin * (PAIRS ? 8 * Mma<K>::PS : 4 * SW);
+  a.ga += 4 * begin;
+  a.y -= 4 * begin * SW;
+  a.gb -= 4 * begin;
   grp.clear();
   grp.template terms<PAIRS>(n, a);
   int v[NT][2][NB], hi[NT][2][NB], top[NT][2] = {};
@@ -831,6 +978,8 @@ __global__ void __launch_bounds__(mma_max_threads(K)) dag_mma_kernel(DagArgs a) 
       at.flat = is_flat<K>(f);
       at.gmax = at.flat ? f.gmax : 0;
       at.every = drain_terms<K>(f);
+      if (tid == 0)
+        *reinterpret_cast<Range*>(sm + kRangeWord) = Range{f.x0, f.x1, f.y0, f.y1, f.spread >= 4 * L};
       form_rows<K, PAIRS>(buf + lay.x, d + 1, buf + lay.y, my, d + 1, at.flat, at.gmax);
       __syncthreads();
       const int base = 4 * (kMiscWords + cur * lay.words);
@@ -942,6 +1091,11 @@ __global__ void __launch_bounds__(mma_max_threads(K)) dag_mma_tiled_kernel(DagAr
         // groups of consecutive column tiles, longest first, in passes of one per warp
         const int gsz = min(NT, (ntiles + warps - 1) / warps);
         const int ngroups = (ntiles + gsz - 1) / gsz;
+        // Only chunks of terms that meet nonzero coefficients in a column of the tile are staged
+        // (8 products of 16, d = 1023, k = 10, inputs of degree 1: integer pipe 3.1 ms, all
+        // chunks 8.8 ms, here 2.8 ms).
+        volatile Range* range = reinterpret_cast<volatile Range*>(sm + kRangeWord);
+        tile_range(gX, conv ? gY : gY + d, conv ? 1 : -1, terms, c0);
         for (int p0 = 0; p0 < ngroups; p0 += warps) {
           Group<K> grp;
           const int o = (p0 + warp) * gsz;
@@ -969,6 +1123,7 @@ __global__ void __launch_bounds__(mma_max_threads(K)) dag_mma_tiled_kernel(DagAr
           int held = 0;  // terms since the last carry
           for (int i0 = 0; i0 < terms; i0 += XR) {
             const int xn = min(XR, terms - i0);
+            if (i0 + xn <= range->x0 || i0 >= range->x1) continue;
             // the column rows those terms meet: [y0, y1)
             const int y0 = max(0, c0 - (i0 + xn - 1)), y1 = min(d + 1, c0 + jn - i0);
             __syncthreads();  // the rows staged before are no longer read
@@ -976,7 +1131,7 @@ __global__ void __launch_bounds__(mma_max_threads(K)) dag_mma_tiled_kernel(DagAr
             stage_rows<K, 2 * M::PS, 2>(buf + lay.x + 2 * kPairLead, mx, xs, S, i0, xn, false);
             copies_wait();
             __syncthreads();
-            const Found f = split_metas(mx, ga, xn, my, gb, y1 - y0);
+            const Found f = split_chunk(mx, ga, xn, my, gb, y1 - y0);
             Terms at{};
             at.flat = is_flat<K>(f);
             at.gmax = at.flat ? f.gmax : 0;
