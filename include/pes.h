@@ -61,7 +61,9 @@ typedef struct pes_batch_s* pes_batch_t;
  * PES_ARITH_AUTO takes the integer pipe, or, for polynomials with many products a
  * layer at k >= 4 and degrees from 56 to 256 on, integer digits of 18 or 20 bits on the
  * tensor cores (reported as PES_ARITH_INT).  The choice depends on the sizes of the
- * monomials, k and d: all plans of one polynomial make the same. */
+ * monomials, k and d: all plans of one polynomial make the same, but for one (or a batch)
+ * whose series, up to 1.54 times as long in that form, do not fit the device memory: it
+ * takes the integer pipe. */
 enum { PES_ARITH_AUTO = -1, PES_ARITH_FP64 = 0, PES_ARITH_INT = 1 };
 
 typedef struct {

@@ -761,9 +761,25 @@ extern "C" pes_status pes_plan_system(int32_t P, const int32_t* poly_ptr, const 
 }
 
 namespace {
-pes_status plan_impl(const int32_t* supp_ptr, const int32_t* supp_idx, const int32_t* supp_exp, int32_t N, int32_t n,
-                     int32_t d, int32_t k, const pes_options* opt, pes_plan_t* out, bool complex_series,
-                     const std::vector<int32_t>* poly_ptr) {
+// `build(options, &tensor)` with the caller's options; a plan that the automatic
+// arithmetic put on the tensor cores (`tensor`) and whose series, up to 1.54 times as
+// long in that form, do not fit the device memory is built for the integer pipe instead.
+template <class Build>
+pes_status build_within_memory(const pes_options* opt, Build build) {
+  bool tensor = false;
+  const pes_status s = build(opt, &tensor);
+  if (s != PES_ENOMEM || !tensor || (opt && opt->arith != PES_ARITH_AUTO)) return s;
+  (void)cudaGetLastError();  // the failed allocation's
+  pes_options o;
+  pes_default_options(&o);
+  if (opt) o = *opt;
+  o.arith = PES_ARITH_INT;
+  return build(&o, &tensor);
+}
+
+pes_status plan_build(const int32_t* supp_ptr, const int32_t* supp_idx, const int32_t* supp_exp, int32_t N, int32_t n,
+                      int32_t d, int32_t k, const pes_options* opt, pes_plan_t* out, bool complex_series,
+                      const std::vector<int32_t>* poly_ptr, bool* tensor) {
   if (!out) return fail(PES_EINVAL, "out is NULL");
   *out = nullptr;
   if (!valid_k(k)) return fail(PES_EUNSUPPORTED_K, "k must be one of 1,2,3,4,5,8,10");
@@ -790,6 +806,7 @@ pes_status plan_impl(const int32_t* supp_ptr, const int32_t* supp_idx, const int
   const int32_t S = pes::series_stride(d);
   const int32_t slots = P->with_vjp ? G.n_slots_vjp : G.n_slots;
   o.arith = resolve_arith(k, o.arith, d, sup, poly_ptr, device_optin());
+  *tensor = o.arith == pes::ARITH_MMA;
   const int64_t sstride = pes::ws_slot_words(k, o.arith, S);
   std::vector<pes::InstInfo> insts{{0, sstride, S, d}};
   s = P->ex.init(k, o, insts, static_cast<size_t>(slots) * static_cast<size_t>(sstride));
@@ -958,6 +975,14 @@ pes_status plan_impl(const int32_t* supp_ptr, const int32_t* supp_idx, const int
   }
   *out = P.release();
   return PES_OK;
+}
+
+pes_status plan_impl(const int32_t* supp_ptr, const int32_t* supp_idx, const int32_t* supp_exp, int32_t N, int32_t n,
+                     int32_t d, int32_t k, const pes_options* opt, pes_plan_t* out, bool complex_series,
+                     const std::vector<int32_t>* poly_ptr) {
+  return build_within_memory(opt, [&](const pes_options* o, bool* tensor) {
+    return plan_build(supp_ptr, supp_idx, supp_exp, N, n, d, k, o, out, complex_series, poly_ptr, tensor);
+  });
 }
 }  // namespace
 
@@ -1272,10 +1297,10 @@ extern "C" pes_status pes_plan_batch(int32_t count, const int32_t* n, const int3
   return pes_plan_batch_powers(count, n, N, d, supp_ptr, supp_idx, nullptr, k, opt, out);
 }
 
-extern "C" pes_status pes_plan_batch_powers(int32_t count, const int32_t* n, const int32_t* N, const int32_t* d,
-                                            const int32_t* supp_ptr, const int32_t* supp_idx,
-                                            const int32_t* supp_exp, int32_t k, const pes_options* opt,
-                                            pes_batch_t* out) {
+namespace {
+pes_status batch_build(int32_t count, const int32_t* n, const int32_t* N, const int32_t* d, const int32_t* supp_ptr,
+                       const int32_t* supp_idx, const int32_t* supp_exp, int32_t k, const pes_options* opt,
+                       pes_batch_t* out, bool* tensor) {
   if (!out) return fail(PES_EINVAL, "out is NULL");
   *out = nullptr;
   if (count < 1 || !n || !N || !d || !supp_ptr) return fail(PES_EINVAL, "bad batch arguments");
@@ -1317,6 +1342,7 @@ extern "C" pes_status pes_plan_batch_powers(int32_t count, const int32_t* n, con
     prow += N[b] + 1;
     qidx += sup.ptr.back();
     const int32_t ar = resolve_arith(k, o.arith, d[b], sup, nullptr, optin);
+    *tensor = *tensor || ar == pes::ARITH_MMA;
     const bool tiled = o.tile > 0 || !whole_series_fits(k, ar, d[b], o.threads, optin);
     // default CTA: one lane per coefficient within the cap
     const int32_t T = std::min((2 * ((d[b] + 2) / 2) + 31) / 32 * 32, pes::dag_max_threads(k));
@@ -1419,6 +1445,16 @@ extern "C" pes_status pes_plan_batch_powers(int32_t count, const int32_t* n, con
     for (cudaEvent_t& e : B->ev) PES_CUDA(cudaEventCreate(&e));
   *out = B.release();
   return PES_OK;
+}
+}  // namespace
+
+extern "C" pes_status pes_plan_batch_powers(int32_t count, const int32_t* n, const int32_t* N, const int32_t* d,
+                                            const int32_t* supp_ptr, const int32_t* supp_idx,
+                                            const int32_t* supp_exp, int32_t k, const pes_options* opt,
+                                            pes_batch_t* out) {
+  return build_within_memory(opt, [&](const pes_options* o, bool* tensor) {
+    return batch_build(count, n, N, d, supp_ptr, supp_idx, supp_exp, k, o, out, tensor);
+  });
 }
 
 extern "C" void pes_batch_destroy(pes_batch_t batch) { delete batch; }
