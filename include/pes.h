@@ -58,16 +58,18 @@ typedef struct pes_batch_s* pes_batch_t;
  * digit products of every output coefficient exactly and round the sum once to
  * k limbs (24-bit digits on the FP64 FMA pipe, 28-bit digits with 32x32->64-bit
  * integer multiply-add); results agree to within the last limb's rounding.
- * PES_ARITH_AUTO takes the integer pipe, or, for polynomials with many products a
- * layer at k >= 4 and degrees from 56 to 256 on, integer digits of 18 or 20 bits on the
- * tensor cores (reported as PES_ARITH_INT).  The choice depends on the sizes of the
- * monomials, k and d: all plans of one polynomial make the same, but for one (or a batch)
- * whose series, up to 1.54 times as long in that form, do not fit the device memory: it
- * takes the integer pipe. */
-enum { PES_ARITH_AUTO = -1, PES_ARITH_FP64 = 0, PES_ARITH_INT = 1 };
+ * PES_ARITH_TENSOR (k = 4, 5, 8 and 10) forms the integer sums on the tensor cores, from
+ * digits of 18 or 20 bits; its outputs differ from PES_ARITH_INT's below the last limb.
+ * PES_ARITH_AUTO takes the integer pipe, or the tensor cores for polynomials with many
+ * products a layer at k >= 4 and degrees from 56 to 256 on.  The choice depends on the
+ * sizes of the monomials, k and d (pes_auto_arith tells it): all plans of one polynomial
+ * make the same, but for one (or a batch) whose series, up to 1.54 times as long on the
+ * tensor cores, do not fit the device memory: it takes the integer pipe.  Plans given one
+ * arithmetic by name give the same bits whatever else they hold. */
+enum { PES_ARITH_AUTO = -1, PES_ARITH_FP64 = 0, PES_ARITH_INT = 1, PES_ARITH_TENSOR = 2 };
 
 typedef struct {
-  int32_t arith;       /* PES_ARITH_AUTO (default), PES_ARITH_FP64 or PES_ARITH_INT */
+  int32_t arith;       /* PES_ARITH_AUTO (default), PES_ARITH_FP64, PES_ARITH_INT or PES_ARITH_TENSOR */
   int32_t threads;     /* threads per CTA of the convolution kernel (a multiple of 32), 0 = automatic.
                           Integer pipe: the lanes are spread evenly over the coefficient pairs (j, d-j),
                           automatic = two lanes per pair (one per output coefficient; three at k = 10),
@@ -157,8 +159,8 @@ pes_status pes_plan_complex(const int32_t* supp_ptr, const int32_t* supp_idx, co
  * supp_exp may be NULL) plus its own constant series.  All polynomials share
  * the input series and one job table; the products of every monomial are the
  * ones its own plan would compute, so every output is bit-identical to a plan
- * of that polynomial alone in the same arithmetic (PES_ARITH_AUTO takes the tensor
- * cores for a system when it would for each of its polynomials).  Evaluate with pes_eval_system (pes_eval_grad is
+ * of that polynomial alone in the same arithmetic (pes_get_plan_arith: PES_ARITH_AUTO takes
+ * the tensor cores for a system when it would for each of its polynomials).  Evaluate with pes_eval_system (pes_eval_grad is
  * pes_eval_system with PES_LAYOUT_SERIES); pes_vjp takes one upstream series
  * per polynomial.
  *   P >= 1, poly_ptr: P+1 non-decreasing entries, poly_ptr[0] == 0.
@@ -254,7 +256,8 @@ typedef struct {
   int32_t grid;            /* persistent CTAs of the convolution kernel */
   int32_t threads;         /* threads per CTA */
   int32_t smem_bytes;      /* dynamic shared memory per CTA */
-  int32_t arith;           /* PES_ARITH_FP64 or PES_ARITH_INT: the pipe the plan uses */
+  int32_t arith;           /* PES_ARITH_FP64 or PES_ARITH_INT, whose digits the sums are rounded and
+                              exchanged in (also on the tensor cores: pes_get_plan_arith) */
   int32_t staging;         /* staging depth in use (1 or 2) */
   int32_t split;           /* parts per convolution job in use */
   int32_t complex_series;  /* 1 for a plan of pes_plan_complex */
@@ -263,6 +266,15 @@ typedef struct {
 } pes_plan_info;
 
 pes_status pes_get_plan_info(pes_plan_t plan, pes_plan_info* info);
+
+/* The arithmetic PES_ARITH_AUTO takes for a polynomial of N monomials with row pointers
+ * supp_ptr (as pes_plan), degree d and k limbs: PES_ARITH_INT or PES_ARITH_TENSOR.  Host
+ * only. */
+pes_status pes_auto_arith(const int32_t* supp_ptr, int32_t N, int32_t d, int32_t k, int32_t* arith);
+
+/* The arithmetic of a plan, to give to others that have to agree with it: PES_ARITH_FP64,
+ * PES_ARITH_INT or PES_ARITH_TENSOR. */
+pes_status pes_get_plan_arith(pes_plan_t plan, int32_t* arith);
 
 /* ---- one polynomial split over ranks ---------------------------------------------
  *
@@ -275,8 +287,8 @@ pes_status pes_get_plan_info(pes_plan_t plan, pes_plan_info* info);
  * pes_partial_sums, an all-reduce (sum) of the digit sums and pes_round_sums,
  * every rank obtains the value and gradient that one plan of the whole polynomial
  * computes, bit for bit, if all of them are given the same arithmetic
- * (PES_ARITH_INT or PES_ARITH_FP64; PES_ARITH_AUTO goes by the monomials of each plan,
- * and differs below the last limb's rounding): the addition stage sums the contributions of every
+ * (that of the whole polynomial, pes_auto_arith; PES_ARITH_AUTO goes by the monomials of
+ * each plan, and differs below the last limb's rounding): the addition stage sums the contributions of every
  * output coefficient on the largest grid among them and rounds once, and both
  * the maximum and the sum of integers are exact in any order.  (A sum of the
  * ranks' rounded k-double limbs in floating point would not be.)
@@ -317,7 +329,8 @@ pes_status pes_round_sums(pes_plan_t plan, const int32_t* grids, const int64_t* 
                           void* stream);
 
 /* The same rounding on the host (host buffers; no GPU needed), for k limbs and
- * the digits of `arith` (PES_ARITH_INT or PES_ARITH_FP64), n variables, degree d. */
+ * the digits of `arith` (PES_ARITH_FP64, or PES_ARITH_INT or PES_ARITH_TENSOR, which
+ * exchange the same digits), n variables, degree d. */
 pes_status pes_round_sums_host(int32_t k, int32_t arith, int32_t n, int32_t d, const int32_t* grids,
                                const int64_t* acc, double* value, double* grad);
 

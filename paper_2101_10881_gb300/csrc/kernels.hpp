@@ -114,6 +114,8 @@ __host__ __device__ constexpr int dag_max_regs(int k, bool intv) {
 __host__ __device__ constexpr bool dag_has_narrow(int k, bool intv) { return intv && k <= 2; }
 constexpr int kNarrowThreads = 256;  // widest CTA of the narrow instantiation
 constexpr int kNarrowCtas = 4;       // CTAs per SM its launch bounds declare
+// k with tensor-core kernels.
+__host__ __device__ constexpr bool mma_has(int k) { return k == 4 || k == 5 || k == 8 || k == 10; }
 // The most the tensor-core kernels launch with (their accumulators' registers: 168 a
 // thread at k = 8 and 10, 128 at k = 5, 96 at k = 4); a wider request runs with this many.
 __host__ __device__ constexpr int mma_max_threads(int k) { return k >= 8 ? 384 : k >= 5 ? 512 : 640; }

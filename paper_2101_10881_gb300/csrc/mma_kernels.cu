@@ -1193,7 +1193,7 @@ constexpr size_t kPairsBytes = 224 * 1024;
 // coefficient's slices fill too little of a 16-slice block (20 % slower at k = 2, d = 152).
 // Degrees whose whole series fit in shared memory only as 28-bit digits stay there.
 bool mma_takes(int k, int d, const int32_t* supp_ptr, int32_t m0, int32_t m1, bool whole, size_t optin) {
-  if (m0 >= m1 || (k != 4 && k != 5 && k < 8)) return false;
+  if (m0 >= m1 || !mma_has(k)) return false;
   if (d < (k == 4 ? 136 : k == 5 ? 256 : k == 8 ? 72 : 56)) return false;
   if (whole && mma_smem_bytes(k, d, 1) > optin) return false;
   // products and layers of the monomials (3 n - 3 and n of one of n >= 2 variables)

@@ -134,6 +134,11 @@ int32_t resolve_arith(int32_t k, int32_t requested, int32_t d, const pes::Suppor
 // the window of the second they meet).
 constexpr int32_t kStagedRows = 128;
 
+// Shared memory a CTA may take on this architecture (sm_103a).
+constexpr int kOptinBytes = 227 * 1024;
+static_assert(PES_ARITH_FP64 == pes::ARITH_FP64 && PES_ARITH_INT == pes::ARITH_INT && PES_ARITH_TENSOR == pes::ARITH_MMA,
+              "the arithmetics of the interface are the library's");
+
 int device_optin() {
   int dev = 0, optin = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return 0;
@@ -503,11 +508,13 @@ struct Exec {
   }
 };
 
-pes_status parse_options(const pes_options* opt, pes_options& o) {
+pes_status parse_options(const pes_options* opt, int32_t k, pes_options& o) {
   pes_default_options(&o);
   if (opt) o = *opt;
-  if (o.arith != PES_ARITH_AUTO && o.arith != PES_ARITH_FP64 && o.arith != PES_ARITH_INT)
-    return fail(PES_EINVAL, "arith must be -1, 0 or 1");
+  if (o.arith != PES_ARITH_AUTO && o.arith != PES_ARITH_FP64 && o.arith != PES_ARITH_INT && o.arith != PES_ARITH_TENSOR)
+    return fail(PES_EINVAL, "arith must be -1, 0, 1 or 2");
+  if (o.arith == PES_ARITH_TENSOR && !pes::mma_has(k))
+    return fail(PES_EINVAL, "the tensor cores take k = 4, 5, 8 and 10");
   if (o.threads < 0 || o.threads > 1024 || o.threads % 32 != 0)
     return fail(PES_EINVAL, "threads must be 0 (automatic) or a multiple of 32 up to 1024");
   if (o.ctas_per_sm < 0) return fail(PES_EINVAL, "ctas_per_sm must be >= 0");
@@ -786,7 +793,7 @@ pes_status plan_build(const int32_t* supp_ptr, const int32_t* supp_idx, const in
   if (d < 0) return fail(PES_EINVAL, "d must be >= 0");
   if (d > pes::kMaxDegree) return fail(PES_EUNSUPPORTED_SIZE, "d must be <= " + std::to_string(pes::kMaxDegree));
   pes_options o;
-  pes_status s = parse_options(opt, o);
+  pes_status s = parse_options(opt, k, o);
   if (s != PES_OK) return s;
   pes::Supports sup;
   s = build_supports(supp_ptr, supp_idx, N, n, sup, supp_exp);
@@ -1117,7 +1124,8 @@ extern "C" pes_status pes_round_sums(pes_plan_t plan, const int32_t* grids, cons
 extern "C" pes_status pes_round_sums_host(int32_t k, int32_t arith, int32_t n, int32_t d, const int32_t* grids,
                                           const int64_t* acc, double* value, double* grad) {
   if (!valid_k(k)) return fail(PES_EUNSUPPORTED_K, "k must be one of 1,2,3,4,5,8,10");
-  if (arith != pes::ARITH_INT && arith != pes::ARITH_FP64) return fail(PES_EINVAL, "arith must be 0 or 1");
+  if (arith != PES_ARITH_INT && arith != PES_ARITH_FP64 && arith != PES_ARITH_TENSOR)
+    return fail(PES_EINVAL, "arith must be 0, 1 or 2");
   if (n < 1 || d < 0 || d > pes::kMaxDegree || !grids || !acc || !value || !grad)
     return fail(PES_EINVAL, "bad sizes or NULL buffer");
   pes::RoundArgs a{grids, reinterpret_cast<const long long*>(acc), value, grad, n, d};
@@ -1306,7 +1314,7 @@ pes_status batch_build(int32_t count, const int32_t* n, const int32_t* N, const 
   if (count < 1 || !n || !N || !d || !supp_ptr) return fail(PES_EINVAL, "bad batch arguments");
   if (!valid_k(k)) return fail(PES_EUNSUPPORTED_K, "k must be one of 1,2,3,4,5,8,10");
   pes_options o;
-  pes_status s = parse_options(opt, o);
+  pes_status s = parse_options(opt, k, o);
   if (s != PES_OK) return s;
   std::unique_ptr<pes_batch_s> B(new (std::nothrow) pes_batch_s());
   if (!B) return fail(PES_ENOMEM, "batch");
@@ -1568,6 +1576,26 @@ extern "C" pes_status pes_batch_check(pes_batch_t batch, void* stream) {
     pes_status s = G->ex.check(G->stream);
     if (s != PES_OK) return s;
   }
+  return PES_OK;
+}
+
+extern "C" pes_status pes_auto_arith(const int32_t* supp_ptr, int32_t N, int32_t d, int32_t k, int32_t* arith) {
+  if (!arith) return fail(PES_EINVAL, "arith is NULL");
+  if (!valid_k(k)) return fail(PES_EUNSUPPORTED_K, "k must be one of 1,2,3,4,5,8,10");
+  if (N < 0 || d < 0 || d > pes::kMaxDegree || (N > 0 && !supp_ptr)) return fail(PES_EINVAL, "bad sizes or NULL pointer");
+  for (int32_t m = 0; m < N; ++m)
+    if (supp_ptr[m + 1] <= supp_ptr[m]) return fail(PES_EINVAL, "empty monomial " + std::to_string(m));
+  pes::Supports sup;
+  sup.N = N;
+  sup.ptr.assign(1, 0);
+  if (N > 0) sup.ptr.assign(supp_ptr, supp_ptr + N + 1);
+  *arith = resolve_arith(k, PES_ARITH_AUTO, d, sup, nullptr, kOptinBytes);
+  return PES_OK;
+}
+
+extern "C" pes_status pes_get_plan_arith(pes_plan_t plan, int32_t* arith) {
+  if (!plan || !arith) return fail(PES_EINVAL, "NULL argument");
+  *arith = plan->ex.arith;
   return PES_OK;
 }
 

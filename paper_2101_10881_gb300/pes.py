@@ -22,7 +22,7 @@ LIB_PATH = os.path.join(_HERE, "_build", "libpes.so")
 PES_OK = 0
 STATUS = {0: "PES_OK", 1: "PES_EINVAL", 2: "PES_EUNSUPPORTED_K", 3: "PES_ENOMEM", 4: "PES_ECUDA",
           5: "PES_ETIMEOUT", 6: "PES_EINTERNAL", 7: "PES_EUNSUPPORTED_SIZE"}
-ARITH = {"auto": -1, "fp64": 0, "int": 1}
+ARITH = {"auto": -1, "fp64": 0, "int": 1, "tensor": 2}
 
 # every symbol that include/pes.h declares
 EXPORTS = ("pes_default_options", "pes_plan", "pes_plan_ex", "pes_plan_powers", "pes_plan_complex", "pes_plan_destroy",
@@ -34,7 +34,7 @@ EXPORTS = ("pes_default_options", "pes_plan", "pes_plan_ex", "pes_plan_powers", 
            "pes_md_binary", "pes_md_costs", "pes_fp64_peak", "pes_int_peak", "pes_jobc_stats", "pes_jobc_jobs",
            "pes_jobc_add_levels", "pes_jobc_add_terms", "pes_selftest_timeout", "pes_eval_grad_static", "pes_status_string",
            "pes_last_error", "pes_shard_range", "pes_partial_grids", "pes_partial_sums", "pes_round_sums",
-           "pes_round_sums_host")
+           "pes_round_sums_host", "pes_auto_arith", "pes_get_plan_arith")
 
 
 class PesError(RuntimeError):
@@ -135,6 +135,8 @@ def lib():
                 "pes_partial_sums": (i32, [vp, vp, vp, vp]),
                 "pes_round_sums": (i32, [vp, vp, vp, vp, vp, vp]),
                 "pes_round_sums_host": (i32, [i32, i32, i32, i32, ip32, ip64, dp, dp]),
+                "pes_auto_arith": (i32, [ip32, i32, i32, i32, ip32]),
+                "pes_get_plan_arith": (i32, [vp, ip32]),
                 "pes_status_string": (ctypes.c_char_p, [i32]),
                 "pes_last_error": (ctypes.c_char_p, []),
             }
@@ -196,6 +198,18 @@ def shard_range(supports, world, rank):
     _check(lib().pes_shard_range(_ip32(ptr), len(supports), int(world), int(rank), ctypes.byref(b), ctypes.byref(e)),
            "pes_shard_range")
     return b.value, e.value
+
+
+def auto_arith(supports, d, k):
+    """The arithmetic ("int" or "tensor") that arith="auto" takes for a polynomial (pes_auto_arith)."""
+    ptr, _ = csr(supports)
+    a = ctypes.c_int32()
+    _check(lib().pes_auto_arith(_ip32(ptr), len(supports), int(d), int(k), ctypes.byref(a)), "pes_auto_arith")
+    return _arith_name(a.value)
+
+
+def _arith_name(value):
+    return next(name for name, v in ARITH.items() if v == value)
 
 
 def round_sums_host(k, n, d, grids, acc, arith="int"):
@@ -380,6 +394,13 @@ class Plan:
         pi = PlanInfo()
         _check(lib().pes_get_plan_info(self._h, ctypes.byref(pi)), "pes_get_plan_info")
         return pi.as_dict()
+
+    def arith(self):
+        """The plan's arithmetic: "fp64", "int" or "tensor" (info() counts in the digits of "int" for both of the
+        latter)."""
+        a = ctypes.c_int32()
+        _check(lib().pes_get_plan_arith(self._h, ctypes.byref(a)), "pes_get_plan_arith")
+        return _arith_name(a.value)
 
 
 LAYOUTS = {"series": 0, "matrix": 1}

@@ -2,9 +2,9 @@
 below the largest) are left out by the tensor-core kernels: same results as the integer pipe
 from every pattern of zeros and of falling magnitudes, and less time for short series.
 
-Both pipes drop less than 2^-(53 k + 8) of the product of the largest coefficients per
-product; 2^24 above a k-double's last bit leaves room for sums over a few hundred terms and
-monomials and for the cancellation between them."""
+Both pipes drop at most 2^-(53 k - 1) of the product of the largest coefficients per product;
+2^24 above a k-double's last bit leaves room for sums over a few hundred terms and monomials
+and for the cancellation between them."""
 import itertools
 
 import numpy as np
