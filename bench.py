@@ -696,7 +696,7 @@ def shard_measure(args, dev, world, rank, prob, ops_step, flush):
     sp.plan.check()
     ms = max_over_ranks(statistics.mean(times), world)
     return {"workload": "the headline polynomial split over the ranks by monomials", "ranks": world,
-            "monomials_this_rank": sp.m_end - sp.m_begin, "ms_per_step": ms,
+            "monomials_this_rank": sp.m_end - sp.m_begin, "arith_used": sp.plan.arith(), "ms_per_step": ms,
             "value": ops_step / (ms * 1e-3) / 1e12, "unit": UNIT, "scaling": "strong",
             "exchange": "all-reduce max of int32 grids, all-reduce sum of int64 digit sums"}
 

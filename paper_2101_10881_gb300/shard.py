@@ -8,8 +8,9 @@ integer arrays through torch.distributed: the largest grid of every output
 coefficient (all-reduce, maximum) and the exact digit sums on those grids
 (all-reduce, sum).  Both are exact in any order, so every rank rounds the
 same sums once and obtains, bit for bit, what one plan of the whole
-polynomial gives in the same arithmetic (arith="int" here, unless another is asked for).  A floating-point all-reduce of the rounded k-double limbs
-would not be exact.
+polynomial gives: every rank takes the arithmetic that the whole polynomial's
+plan would.  A floating-point all-reduce of the rounded k-double limbs would
+not be exact.
 
 Argument marshalling and collectives only: the products, sums and rounding run
 in libpes's kernels (include/pes.h, pes_partial_grids / pes_partial_sums /
@@ -31,8 +32,9 @@ class ShardPlan:
         self.supports = [list(s) for s in supports[self.m_begin:self.m_end]]
         ex = None if exponents is None else [list(e) for e in exponents[self.m_begin:self.m_end]]
         self.n, self.d, self.k = int(n), int(d), int(k)
-        # the automatic arithmetic goes by a plan's monomials: one form on every rank
-        opts.setdefault("arith", "int")
+        # the automatic arithmetic goes by a plan's monomials: here by the whole polynomial's
+        if opts.get("arith", "auto") in ("auto", pes.ARITH["auto"]):
+            opts["arith"] = pes.auto_arith(supports, d, k)
         self.plan = pes.Plan(self.supports, n, d, k, exponents=ex, with_vjp=False, **opts)
 
     def coeff_of(self, coeff):
