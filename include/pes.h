@@ -61,7 +61,8 @@ typedef struct pes_batch_s* pes_batch_t;
  * PES_ARITH_TENSOR (k = 4, 5, 8 and 10) forms the integer sums on the tensor cores, from
  * digits of 18 or 20 bits; its outputs differ from PES_ARITH_INT's below the last limb.
  * PES_ARITH_AUTO takes the integer pipe, or the tensor cores for polynomials with many
- * products a layer at k >= 4 and degrees from 56 to 256 on.  The choice depends on the
+ * products a layer: at k = 10 and 8 from degrees 56 and 72 on, at k = 4 from 136 on, at
+ * k = 5 between 256 and 279.  The choice depends on the
  * sizes of the monomials, k and d (pes_auto_arith tells it): all plans of one polynomial
  * make the same, but for one (or a batch) whose series, up to 1.54 times as long on the
  * tensor cores, do not fit the device memory: it takes the integer pipe.  Plans given one

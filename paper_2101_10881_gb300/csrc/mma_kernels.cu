@@ -1179,23 +1179,41 @@ constexpr size_t kPairsBytes = 224 * 1024;
 
 }  // namespace
 
+bool mma_pairs(int k, int dmax) {
+  return 4 * static_cast<size_t>(kMiscWords + buf_layout(slice_digits(k), mma_stride(k), dmax + 1, dmax + 1, true).words) <=
+         kPairsBytes;
+}
+
 // The line is the work of an average layer in terms (of one coefficient with one column
 // tile): a job's passes around its products (fragment pairs, grids, carries, fewer warps in
 // flight per job) take about 10 us however short it is, so a table needs layers wide enough
-// to keep every SM on several jobs.  Start of the integer pipe -> here, us:
-//   k = 10: 20 k terms 347 -> 392; 49 k 1047 -> 1095; 315 k 4435 -> 3356; 590 k 10400 -> 6340
-//   k = 8:  20 k 277 -> 357; 82 k 451 -> 501; 192 k 180 -> 136 (conv), exponential series
-//           139 -> 168; 314 k 253 -> 170, 197 -> 175; 454 k 1510 -> 1112
-//   k = 4:  117 k 317 -> 432; 184 k 332 -> 480; 420 k 327 -> 320; 612 k 5959 -> 5391;
-//           839 k 214 -> 154, exponential 179 -> 171; 12.5 M 5540 -> 4110
-// Series whose terms lie on grids far apart (the exponential's) take the general loop: there
-// the two sides meet near d = 50 (k = 10), 72 (k = 8), 140 (k = 4), 256 (k = 5).  At k <= 3 a
-// coefficient's slices fill too little of a 16-slice block (20 % slower at k = 2, d = 152).
-// Degrees whose whole series fit in shared memory only as 28-bit digits stay there.
+// to keep every SM on several jobs, and more of them where the staged series leave an SM one
+// CTA.  At k <= 3 a coefficient's slices fill too little of a 16-slice block (20 % slower at
+// k = 2, d = 152).  Degrees whose whole series fit in shared memory only as 28-bit digits
+// stay there, and so do those of k = 4 and 5 with one CTA an SM, but the widest of k = 4.
+//
+// Integer pipe's time over this form's, 7226 random polynomials (monomials of 2 to 16
+// variables), tenth percentile / median for uniform series; exponential ones with
+// coefficients of degree 0; coefficients falling by 2 bits a degree:
+//   k = 10, d 56-253, work 250-330 k   1.14 / 1.32   1.04 / 1.17   0.98 / 1.13
+//           d 254-471, 400-500 k       1.17 / 1.35   1.34 / 1.55   1.02 / 1.15
+//           tiles, 500-750 k           1.33 / 1.43   1.35 / 1.60   (zeros from d = 450 on)
+//   k = 8,  d 72-258, 330-400 k        1.12 / 1.23   0.99 / 1.10   0.94 / 1.07
+//           d 259-507, 750-1120 k      1.18 / 1.40   1.31 / 1.65   1.01 / 1.20
+//           tiles, 1.75-3.25 M         1.05 / 1.25   1.41 / 1.85
+//   k = 4,  d 136-199, 640-800 k       1.10 / 1.16   1.03 / 1.08   0.93 / 1.04
+//           d 200-336, 1.2-1.8 M       1.19 / 1.33   1.25 / 1.47   1.00 / 1.13
+//           d 337-660, 2.8-5.2 M       1.25 / 1.32   1.45 / 1.80   0.98 / 1.14
+//           tiles, 640-800 k           1.05 / 1.10   1.77 / 2.20
+//   k = 5,  d 256-279, 1.2-1.8 M       1.18 / 1.37   1.40 / 1.46   1.04 / 1.16
+// and below the lines: k = 4, d 200-336, 400-640 k 0.88 / 0.98, d 337-660, 0.4-1.8 M 0.80 /
+// 0.97; k = 5, d 280-556 0.80 / 0.95, tiles 0.90 / 0.97; k = 8, d 259-507, 250-400 k 0.93 /
+// 1.05, tiles of exponential series 0.71 / 0.78; one word a digit instead of pairs (no room
+// for them) 0.57 to 0.9 at every k.
 bool mma_takes(int k, int d, const int32_t* supp_ptr, int32_t m0, int32_t m1, bool whole, size_t optin) {
   if (m0 >= m1 || !mma_has(k)) return false;
   if (d < (k == 4 ? 136 : k == 5 ? 256 : k == 8 ? 72 : 56)) return false;
-  if (whole && mma_smem_bytes(k, d, 1) > optin) return false;
+  if (whole && (mma_smem_bytes(k, d, 1) > optin || !mma_pairs(k, d))) return false;
   // products and layers of the monomials (3 n - 3 and n of one of n >= 2 variables)
   int64_t jobs = 0;
   int32_t layers = 1;
@@ -1206,12 +1224,16 @@ bool mma_takes(int k, int d, const int32_t* supp_ptr, int32_t m0, int32_t m1, bo
   }
   const double tiles = (d + 8) / 8, terms = 0.5 * (d + 1);
   const double work = static_cast<double>(jobs) / layers * tiles * terms;
-  return work >= (k >= 8 ? 250e3 : 400e3);
-}
-
-bool mma_pairs(int k, int dmax) {
-  return 4 * static_cast<size_t>(kMiscWords + buf_layout(slice_digits(k), mma_stride(k), dmax + 1, dmax + 1, true).words) <=
-         kPairsBytes;
+  const bool two = 2 * (mma_smem_bytes(k, d, 1) + 1024) <= 228 * 1024;  // two CTAs fit an SM
+  constexpr double kNever = 1e30;
+  double least = kNever;
+  switch (k) {
+    case 4: least = !whole ? 640e3 : !two ? 2.8e6 : d < 173 ? 640e3 : 3.7e3 * d; break;
+    case 5: least = !whole || !two ? kNever : d < 266 ? 750e3 + 45e3 * (d - 256) : 1.2e6; break;
+    case 8: least = !whole ? 1.75e6 : two ? 350e3 : 750e3; break;
+    case 10: least = !whole ? 600e3 : two ? 250e3 : 400e3; break;
+  }
+  return work >= least;
 }
 
 void* mma_kernel(int k, bool tiled, int dmax) {

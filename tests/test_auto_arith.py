@@ -22,6 +22,23 @@ def test_wide_and_narrow_polynomials():
     assert pes.auto_arith([], 152, 10) == "int"
 
 
+# degree and products of two variables on either side of the line, or no line at all
+LINES = [(10, 100, 254), (10, 300, 47), (10, 600, 18), (8, 100, 356), (8, 300, 88), (8, 700, 38), (4, 150, 298),
+         (4, 300, 130), (4, 400, 183), (4, 1100, 6), (5, 256, 118), (5, 275, 166)]
+NEVER = [(10, 55), (8, 71), (8, 520), (4, 135), (4, 700), (5, 255), (5, 300), (5, 900), (3, 152), (2, 152), (1, 152)]
+
+
+@pytest.mark.parametrize("k,d,N", LINES)
+def test_lines(k, d, N):
+    assert pes.auto_arith([[0, 1]] * (N - 1), d, k) == "int"
+    assert pes.auto_arith([[0, 1]] * N, d, k) == "tensor"
+
+
+@pytest.mark.parametrize("k,d", NEVER)
+def test_degrees_that_stay_on_the_integer_pipe(k, d):
+    assert pes.auto_arith([[0, 1]] * 50000, d, k) == "int"
+
+
 def test_arguments_checked_on_host():
     L = pes.lib()
     ptr = np.array([0, 2, 2], dtype=np.int32)

@@ -19,7 +19,7 @@ def torch():
 
 @pytest.mark.parametrize("batch", [False, True])
 def test_falls_back_to_the_integer_pipe(torch, batch):
-    k, d, n = 5, 300, 180
+    k, d, n = 5, 270, 200
     supp = [list(s) for s in itertools.combinations(range(n), 2)]
     gen = torch.Generator(device="cuda")
     gen.manual_seed(1)
