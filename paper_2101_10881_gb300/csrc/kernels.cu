@@ -1650,8 +1650,8 @@ void* dag_fn(bool tiled, bool narrow) {
   return reinterpret_cast<void*>(&dag_kernel<K, INTV>);
 }
 
-void* dag_kernel_ptr(int k, int arith, bool tiled, bool narrow, int dmax) {
-  if (arith == ARITH_MMA) return mma_kernel(k, tiled, dmax);
+void* dag_kernel_ptr(int k, int arith, bool tiled, bool narrow) {
+  if (arith == ARITH_MMA) return mma_kernel(k, tiled);
   const bool iv = arith == ARITH_INT;
   switch (k) {
     case 1: return iv ? dag_fn<1, true>(tiled, narrow) : dag_fn<1, false>(tiled, narrow);
@@ -1688,7 +1688,7 @@ size_t dag_tiled_smem_bytes(int k, int arith, int tile, int xrows) {
 // The dynamic shared-memory limit is a property of the kernel function on a
 // device, shared by every plan: raise it, never lower it, so that a plan built
 // later for a smaller degree cannot break the launches of an earlier one.
-cudaError_t dag_prepare(int k, int arith, size_t smem, int dmax, bool tiled) {
+cudaError_t dag_prepare(int k, int arith, size_t smem, bool tiled) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
@@ -1696,7 +1696,7 @@ cudaError_t dag_prepare(int k, int arith, size_t smem, int dmax, bool tiled) {
   static std::map<std::pair<int, void*>, size_t> granted;
   std::lock_guard<std::mutex> lock(mu);
   for (bool narrow : {false, true}) {  // the same kernel unless k <= 2 whole-series integer
-    void* fn = dag_kernel_ptr(k, arith, tiled, narrow, dmax);
+    void* fn = dag_kernel_ptr(k, arith, tiled, narrow);
     if (!fn) return cudaErrorInvalidValue;
     size_t& cur = granted[std::make_pair(dev, fn)];
     if (smem <= cur) continue;
@@ -1707,15 +1707,15 @@ cudaError_t dag_prepare(int k, int arith, size_t smem, int dmax, bool tiled) {
   return cudaSuccess;
 }
 
-cudaError_t dag_occupancy(int k, int arith, int threads, size_t smem, int dmax, int* blocks_per_sm, bool tiled) {
-  void* fn = dag_kernel_ptr(k, arith, tiled, narrow_launch(threads), dmax);
+cudaError_t dag_occupancy(int k, int arith, int threads, size_t smem, int* blocks_per_sm, bool tiled) {
+  void* fn = dag_kernel_ptr(k, arith, tiled, narrow_launch(threads));
   if (!fn) return cudaErrorInvalidValue;
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, fn, threads, smem);
 }
 
 cudaError_t launch_dag(const DagArgs& a, int k, int arith, int threads, int grid, cudaStream_t st) {
   const bool tiled = a.tile > 0;
-  void* fn = dag_kernel_ptr(k, arith, tiled, narrow_launch(threads), a.dmax);
+  void* fn = dag_kernel_ptr(k, arith, tiled, narrow_launch(threads));
   if (!fn) return cudaErrorInvalidValue;
   const size_t smem = tiled ? dag_tiled_smem_bytes(k, arith, a.tile, a.xrows)
                             : dag_smem_bytes(k, arith, a.smax, a.dmax, a.depth, threads);

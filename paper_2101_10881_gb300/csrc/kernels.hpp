@@ -163,9 +163,9 @@ inline int32_t add_group_warps(int64_t max_contrib, int64_t items, int32_t nsm) 
   return gw;
 }
 
-// The tensor-core convolution kernel of k for degrees up to dmax (mma_kernels.cu), its
-// shared memory and its threads per CTA.
-void* mma_kernel(int k, bool tiled, int dmax);
+// The tensor-core convolution kernel of k (mma_kernels.cu), its shared memory and its
+// threads per CTA for degrees up to dmax.
+void* mma_kernel(int k, bool tiled);
 size_t mma_smem_bytes(int k, int dmax, int depth);
 int mma_threads(int k, int dmax);
 size_t mma_tiled_smem_bytes(int k, int tile, int xrows);
@@ -182,8 +182,8 @@ cudaError_t launch_add_pair(const AddArgs& a0, int64_t items0, const AddArgs& a1
 cudaError_t launch_round_sums(const RoundArgs& a, int k, int arith, cudaStream_t st);
 // The same rounding on the host (no GPU needed).
 int round_sums_host(int k, int arith, const RoundArgs& a);
-cudaError_t dag_occupancy(int k, int arith, int threads, size_t smem, int dmax, int* blocks_per_sm, bool tiled = false);
-cudaError_t dag_prepare(int k, int arith, size_t smem, int dmax, bool tiled = false);
+cudaError_t dag_occupancy(int k, int arith, int threads, size_t smem, int* blocks_per_sm, bool tiled = false);
+cudaError_t dag_prepare(int k, int arith, size_t smem, bool tiled = false);
 cudaError_t launch_md_binary(int op, int k, const double* x, const double* y, double* out,
                              int64_t count, cudaStream_t st);
 cudaError_t launch_fp64_peak(double* sink, int blocks, int threads, int iters, cudaStream_t st);

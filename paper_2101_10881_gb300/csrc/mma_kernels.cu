@@ -46,9 +46,6 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
-#include <map>
-#include <mutex>
-#include <tuple>
 
 #include "dag_sync.cuh"
 #include "kernels.hpp"
@@ -61,12 +58,12 @@ namespace {
 // Shared memory of one buffer, in words: eight rows of zeros and the column
 // operand's rows behind them, the Toeplitz operand's rows, and the grids of both; the
 // column grids have kPad entries of kZeroGrid on either side (columns before the series
-// have no term there).  PAIRS: a row of the Toeplitz operand holds, for every word u from
+// have no term there).  A row of the Toeplitz operand holds, for every word u from
 // -8 to L - 1, the two fragment words that start at slices 2 u and 2 u + 1 (zeros up to
 // u = -2, which also follow the row before), so that a lane gets both with one 64-bit
 // load; it takes twice the room of the words themselves, which are staged in place first.
-// Without (degrees too large for it), rows of SW words, the fragment words formed as they
-// are read.
+// (One word a digit, the fragment words formed as they are read, for degrees without room
+// for the pairs: 0.57 to 0.9 of the integer pipe's speed, and of the tiles' that take them.)
 constexpr int kPairLead = 8;
 constexpr int kPad = 48;               // > 7 + 8 (NT - 1): how far before the series a group's columns run
 constexpr int kZeroGrid = -(1 << 24);  // staged grid (four times the grid) of a zero coefficient
@@ -74,11 +71,11 @@ constexpr int32_t kZeroMeta = -(1 << 30);  // the meta of a zero coefficient
 struct BufLayout {
   int y, x, ga, gb, mx, my, words;  // (mx, my: the metas as copied)
 };
-__host__ __device__ constexpr BufLayout buf_layout(int L, int sw, int xrows, int yrows, bool pairs) {
+__host__ __device__ constexpr BufLayout buf_layout(int L, int sw, int xrows, int yrows) {
   BufLayout b{};
   b.y = 8 * sw;
   b.x = b.y + (yrows + 1) * sw;  // (a row of zeros, before the Toeplitz operand's coefficient 0 and after the columns)
-  b.ga = b.x + (pairs ? xrows * 2 * (L + kPairLead) + sw : xrows * sw + sw);
+  b.ga = b.x + xrows * 2 * (L + kPairLead) + sw;
   b.gb = b.ga + xrows;
   b.mx = b.gb + kPad + yrows + kPad;
   b.my = b.mx + xrows;
@@ -95,6 +92,9 @@ __host__ __device__ constexpr BufLayout buf_layout(int L, int sw, int xrows, int
 __host__ __device__ constexpr int mma_stride(int k) {
   return k <= 4 ? 36 : k <= 5 ? 44 : 8 * ((slice_digits(k) + 7) / 8) + 4;
 }
+
+constexpr int kMiscWords = 32;
+constexpr int kRangeWord = 8;  // where a Range starts in the misc words
 
 template <int K>
 struct Mma {
@@ -121,11 +121,11 @@ struct Mma {
   static_assert(8 * NB - L <= 8, "the fragments read no further than the zeros after a row of pairs");
   static_assert(SW - L >= 4 && PZ >= 0 && SP >= 0 && SP <= RA, "zeros between the staged coefficients");
   static_assert(kDrain >= 1, "one term must fit the accumulators");
+  static_assert(4 * (kMiscWords + buf_layout(L, SW, kLimit + 1, kLimit + 1).words) > 227 * 1024,
+                "whole series that fit in shared memory are never carried in between");
   static_assert(kPad > 8 * NT, "pads of the column grids");
 };
 
-constexpr int kMiscWords = 32;
-constexpr int kRangeWord = 8;  // where a Range starts in the misc words
 
 // All of the kernels' shared memory: kMiscWords words, then the buffers.  Staged rows
 // and grids are addressed by byte offsets into it (word indices would cost a shift at
@@ -321,9 +321,9 @@ __device__ __forceinline__ bool is_flat(const Found& f) {
 }
 
 // The passes over the staged rows, G lanes a row: the fragment pairs of nx Toeplitz
-// rows (PAIRS), and the ny column rows shifted by gmax minus their grid (`flat`; the
+// rows, and the ny column rows shifted by gmax minus their grid (`flat`; the
 // words behind a row's digits are cleared either way).
-template <int K, bool PAIRS>
+template <int K>
 __device__ __forceinline__ void form_rows(uint32_t* x, int nx, uint32_t* y, const int32_t* my, int ny, bool flat,
                                           int gmax) {
   using M = Mma<K>;
@@ -331,7 +331,7 @@ __device__ __forceinline__ void form_rows(uint32_t* x, int nx, uint32_t* y, cons
   const int p = threadIdx.x % G, r = threadIdx.x / G;
   const int per = blockDim.x / G;
   const bool word = p < L;
-  if constexpr (PAIRS) {
+  {
     uint32_t* at = x + (r * M::PS + kPairLead + p) * 2;
     const int step = per * M::PS * 2;
     const bool follows = p < G - 1;  // (the last lane's shuffle returns its own word)
@@ -474,22 +474,12 @@ struct Group {
   }
 
   // the Toeplitz fragments of the row at xr: word offset 4 (kap - 1), slice rho
-  template <bool PAIRS>
-  __device__ __forceinline__ static void fragments(uint32_t (&A)[2 * NB][2], int xr, int la) {
+  __device__ __forceinline__ static void fragments(uint32_t (&A)[2 * NB][2], int xr) {
 #pragma unroll
     for (int kap = 0; kap < 2 * NB; ++kap) {
-      if constexpr (PAIRS) {
-        const uint2 w = lds2(xr + 32 * (kap - 1));
-        A[kap][0] = w.x;
-        A[kap][1] = w.y;
-      } else {
-        // (words before -4 may belong to the coefficient before: all of them are zeros)
-        const int u = la + 4 * (kap - 1);
-        const uint32_t w0 = lds(xr + 4 * (kap == 0 ? max(u, -4) : u));
-        const uint32_t w1 = lds(xr + 4 * (kap == 0 ? max(u + 1, -4) : u + 1));
-        A[kap][0] = __byte_perm(w0, w1, 0x1032);
-        A[kap][1] = __byte_perm(w0, w1, 0x7610);
-      }
+      const uint2 w = lds2(xr + 32 * (kap - 1));
+      A[kap][0] = w.x;
+      A[kap][1] = w.y;
     }
   }
 
@@ -516,10 +506,10 @@ struct Group {
   }
 
   // The terms i in [i0, i1) of the first NA tiles, every column by its own grid.
-  template <int NA, bool PAIRS>
+  template <int NA>
   __device__ __forceinline__ void run_any(int i0, int i1, const Terms& a, int& left) {
     const int lane = threadIdx.x & 31, la = (lane >> 2) - (lane & 3) - 1, wl = lane & 3;
-    int xr = a.x + (PAIRS ? (i0 * M::PS + kPairLead + la) * 8 : i0 * SW * 4);
+    int xr = a.x + (i0 * M::PS + kPairLead + la) * 8;
     int yr = a.y - i0 * SW * 4, gb = a.gb - i0 * 4;
     const int near = 4 * (a.flat ? PZ : SW - L);
     const int end = a.ga + 4 * i1;
@@ -527,7 +517,7 @@ struct Group {
     for (int ga = a.ga + 4 * i0; ga != end; ga += 4) {
       const int gx = static_cast<int>(lds(ga));
       uint32_t A[2 * NB][2];
-      fragments<PAIRS>(A, xr, la);
+      fragments(A, xr);
 #pragma unroll
       for (int t = 0; t < NA; ++t) {
         // bytes the column is shifted by: 4 for every digit the term lies below the
@@ -551,7 +541,7 @@ struct Group {
         }
         multiply(t, A, Bf);
       }
-      xr += PAIRS ? 8 * M::PS : 4 * SW;
+      xr += 8 * M::PS;
       yr -= 4 * SW;
       gb -= 4;
       if (--left == 0) {
@@ -567,11 +557,11 @@ struct Group {
   // address of a column row is one sum.  The fragments of the next term and the next
   // column rows are loaded while the products of the present ones issue; without that
   // the loads' latency, not the mma, bounds the loop (2 to 4 warps per scheduler).
-  template <int NA, bool PAIRS>
+  template <int NA>
   __device__ __forceinline__ void run_flat(int i0, int i1, int lo, const Terms& a, int& left) {
     const int lane = threadIdx.x & 31, la = (lane >> 2) - (lane & 3) - 1;
-    constexpr int XS = PAIRS ? 8 * M::PS : 4 * SW;
-    int xr = a.x + (PAIRS ? (i0 * M::PS + kPairLead + la) * 8 : i0 * SW * 4);
+    constexpr int XS = 8 * M::PS;
+    int xr = a.x + (i0 * M::PS + kPairLead + la) * 8;
     int yr = a.y - i0 * SW * 4;
     int yt[NA];
 #pragma unroll
@@ -580,7 +570,7 @@ struct Group {
     int ga = a.ga + 4 * i0;
     uint32_t A[2][2 * NB][2], Bf[2][KS][2];
     int yg = yr + max(static_cast<int>(lds(ga)), lo);
-    fragments<PAIRS>(A[0], xr, la);
+    fragments(A[0], xr);
     load(Bf[0], yg + yt[0]);
     for (;;) {
 #pragma unroll
@@ -591,7 +581,7 @@ struct Group {
         xr = more ? xr + XS : xr;
         yr = more ? yr - 4 * SW : yr;
         const int yn = yr + max(static_cast<int>(lds(ga)), lo);
-        fragments<PAIRS>(A[h ^ 1], xr, la);
+        fragments(A[h ^ 1], xr);
 #pragma unroll
         for (int t = 0; t < NA; ++t) {
           load(Bf[(h * NA + t + 1) & 1], t + 1 < NA ? yg + yt[t + 1 < NA ? t + 1 : 0] : yn + yt[0]);
@@ -609,7 +599,6 @@ struct Group {
   }
 
   // Add the terms [0, n[t]) of every tile, n not increasing (tiles without terms last).
-  template <bool PAIRS>
   __device__ __forceinline__ void terms(const int (&n)[NT], const Terms& a) {
     // terms from `from` on take the flat loop
     const int lo = gs_hi - a.gmax - 4 * PZ, hi = gs_lo - a.gmax + 4 * M::RA;
@@ -623,19 +612,19 @@ struct Group {
       from = __reduce_max_sync(0xffffffffu, from);
     }
     int left = a.every, i = 0;
-    segment<NT, PAIRS>(n, i, from, lo, a, left);
+    segment<NT>(n, i, from, lo, a, left);
 #pragma unroll
     for (int t = 0; t < NT; ++t) drain(t);
   }
-  template <int NA, bool PAIRS>
+  template <int NA>
   __device__ __forceinline__ void segment(const int (&n)[NT], int& i, int from, int lo, const Terms& a, int& left) {
     if (n[NA - 1] > i) {
       const int mid = min(max(i, from), n[NA - 1]);
-      if (mid > i) run_any<NA, PAIRS>(i, mid, a, left);
-      if (n[NA - 1] > mid) run_flat<NA, PAIRS>(mid, n[NA - 1], lo, a, left);
+      if (mid > i) run_any<NA>(i, mid, a, left);
+      if (n[NA - 1] > mid) run_flat<NA>(mid, n[NA - 1], lo, a, left);
       i = n[NA - 1];
     }
-    if constexpr (NA > 1) segment<NA - 1, PAIRS>(n, i, from, lo, a, left);
+    if constexpr (NA > 1) segment<NA - 1>(n, i, from, lo, a, left);
   }
 
   // The rows of every tile and column 2 tl + cc as words of one digit and what lies above
@@ -810,7 +799,7 @@ __device__ __forceinline__ void add_rows(const int32_t* xs, const int32_t* ys, i
 // coefficients is read from shared memory for every group: registers are what the term
 // loop has fewest of.  (128 products of 64, k = 10, uniform series: 6.13 ms without the
 // ranges, 6.20 with them.)
-template <int K, bool PAIRS>
+template <int K>
 __device__ __forceinline__ void columns(int d, int o, int nt, Terms a, bool rev, int32_t* zrows, int32_t* zmeta) {
   constexpr int SW = Mma<K>::SW, NT = Mma<K>::NT, NB = Mma<K>::NB;
   const int lane = threadIdx.x & 31, g = lane >> 2, tl = lane & 3;
@@ -854,12 +843,12 @@ __device__ __forceinline__ void columns(int d, int o, int nt, Terms a, bool rev,
   }
 #pragma unroll
   for (int t = 0; t < NT; ++t) n[t] = min(n[t], end) - begin;
-  a.x += begin * (PAIRS ? 8 * Mma<K>::PS : 4 * SW);
+  a.x += begin * 8 * Mma<K>::PS;
   a.ga += 4 * begin;
   a.y -= 4 * begin * SW;
   a.gb -= 4 * begin;
   grp.clear();
-  grp.template terms<PAIRS>(n, a);
+  grp.terms(n, a);
   int v[NT][2][NB], hi[NT][2][NB], top[NT][2] = {};
   grp.words(v, hi);
   grp.carry_words(v, hi, top);
@@ -875,12 +864,12 @@ __device__ __forceinline__ void columns(int d, int o, int nt, Terms a, bool rev,
 // same number of terms.  A correlation is run as a convolution with the series x reversed, and its result stored backwards.  Staging depth 2 claims the next job early
 // and copies its operands into a second buffer, if they are complete, while this one is
 // computed.
-template <int K, bool PAIRS>
+template <int K>
 __global__ void __launch_bounds__(mma_max_threads(K)) dag_mma_kernel(DagArgs a) {
   using M = Mma<K>;
   constexpr int SW = M::SW, NT = M::NT, L = M::L;
   const int tid = threadIdx.x, T = blockDim.x;
-  const BufLayout lay = buf_layout(L, SW, a.dmax + 1, a.dmax + 1, PAIRS);
+  const BufLayout lay = buf_layout(L, SW, a.dmax + 1, a.dmax + 1);
   Claim* next = reinterpret_cast<Claim*>(sm);
   uint32_t* buf0 = sm + kMiscWords;
   const int nbuf = a.depth >= 2 ? 2 : 1;
@@ -924,10 +913,7 @@ __global__ void __launch_bounds__(mma_max_threads(K)) dag_mma_kernel(DagArgs a) 
     int32_t* mx = reinterpret_cast<int32_t*>(buf + lay.mx);
     int32_t* my = reinterpret_cast<int32_t*>(buf + lay.my);
     stage_rows<K, SW, 1>(buf + lay.y, my, conv ? s2 : s1, in.S, 0, in.d + 1, !conv);
-    if constexpr (PAIRS)
-      stage_rows<K, 2 * M::PS, 2>(buf + lay.x + 2 * kPairLead, mx, conv ? s1 : s2, in.S, 0, in.d + 1, false);
-    else
-      stage_rows<K, SW, 1>(buf + lay.x, mx, conv ? s1 : s2, in.S, 0, in.d + 1, false);
+    stage_rows<K, 2 * M::PS, 2>(buf + lay.x + 2 * kPairLead, mx, conv ? s1 : s2, in.S, 0, in.d + 1, false);
   };
 
   bool claimed = false, staged = false;
@@ -980,7 +966,7 @@ __global__ void __launch_bounds__(mma_max_threads(K)) dag_mma_kernel(DagArgs a) 
       at.every = drain_terms<K>(f);
       if (tid == 0)
         *reinterpret_cast<Range*>(sm + kRangeWord) = Range{f.x0, f.x1, f.y0, f.y1, f.spread >= 4 * L};
-      form_rows<K, PAIRS>(buf + lay.x, d + 1, buf + lay.y, my, d + 1, at.flat, at.gmax);
+      form_rows<K>(buf + lay.x, d + 1, buf + lay.y, my, d + 1, at.flat, at.gmax);
       __syncthreads();
       const int base = 4 * (kMiscWords + cur * lay.words);
       at.x = base + 4 * lay.x;
@@ -999,7 +985,7 @@ __global__ void __launch_bounds__(mma_max_threads(K)) dag_mma_kernel(DagArgs a) 
         const int og = q * WT + ((q & 1) ? WT - 1 - wk : wk);
         if (og >= ngroups) continue;
         const int o = og * gsz;  // the o-th longest tile
-        columns<K, PAIRS>(d, o, min(gsz, ntiles - o), at, corr, zrows, zmeta);
+        columns<K>(d, o, min(gsz, ntiles - o), at, corr, zrows, zmeta);
       }
     }
     __syncthreads();
@@ -1026,7 +1012,7 @@ __global__ void __launch_bounds__(mma_max_threads(K)) dag_mma_tiled_kernel(DagAr
   constexpr int SW = M::SW, NT = M::NT, L = M::L;
   const int tid = threadIdx.x, T = blockDim.x, lane = tid & 31, g = lane >> 2, tl = lane & 3;
   const int D = a.tile, XR = a.xrows;
-  const BufLayout lay = buf_layout(L, SW, XR, D + XR, true);
+  const BufLayout lay = buf_layout(L, SW, XR, D + XR);
   Claim* next = reinterpret_cast<Claim*>(sm);
   uint32_t* buf = sm + kMiscWords;
   for (int t = tid; t < lay.words; t += T) buf[t] = 0u;
@@ -1136,7 +1122,7 @@ __global__ void __launch_bounds__(mma_max_threads(K)) dag_mma_tiled_kernel(DagAr
             at.flat = is_flat<K>(f);
             at.gmax = at.flat ? f.gmax : 0;
             at.every = drain_terms<K>(f);
-            form_rows<K, true>(buf + lay.x, xn, buf + lay.y, my, y1 - y0, at.flat, at.gmax);
+            form_rows<K>(buf + lay.x, xn, buf + lay.y, my, y1 - y0, at.flat, at.gmax);
             __syncthreads();
             if (held + xn > M::kLimit) {
               grp.carry(top);
@@ -1153,7 +1139,7 @@ __global__ void __launch_bounds__(mma_max_threads(K)) dag_mma_tiled_kernel(DagAr
             at.y = base + 4 * (lay.y + m * SW + tl);
             at.gb = base + 4 * (lay.gb + kPad + m);
             at.zero = base + 4 * tl;
-            grp.template terms<true>(n, at);
+            grp.terms(n, at);
           }
           int v[NT][2][M::NB], hi[NT][2][M::NB];
           grp.words(v, hi);
@@ -1168,21 +1154,11 @@ __global__ void __launch_bounds__(mma_max_threads(K)) dag_mma_tiled_kernel(DagAr
 }
 
 template <int K>
-void* mma_fn(bool tiled, bool pairs) {
-  if (tiled) return reinterpret_cast<void*>(&dag_mma_tiled_kernel<K>);
-  return pairs ? reinterpret_cast<void*>(&dag_mma_kernel<K, true>) : reinterpret_cast<void*>(&dag_mma_kernel<K, false>);
+void* mma_fn(bool tiled) {
+  return tiled ? reinterpret_cast<void*>(&dag_mma_tiled_kernel<K>) : reinterpret_cast<void*>(&dag_mma_kernel<K>);
 }
-
-// Shared memory a CTA may take for the fragment pairs of its Toeplitz operand; where
-// whole series would need more, they are staged as single words.
-constexpr size_t kPairsBytes = 224 * 1024;
 
 }  // namespace
-
-bool mma_pairs(int k, int dmax) {
-  return 4 * static_cast<size_t>(kMiscWords + buf_layout(slice_digits(k), mma_stride(k), dmax + 1, dmax + 1, true).words) <=
-         kPairsBytes;
-}
 
 // The line is the work of an average layer in terms (of one coefficient with one column
 // tile): a job's passes around its products (fragment pairs, grids, carries, fewer warps in
@@ -1208,12 +1184,11 @@ bool mma_pairs(int k, int dmax) {
 //   k = 5,  d 256-279, 1.2-1.8 M       1.18 / 1.37   1.40 / 1.46   1.04 / 1.16
 // and below the lines: k = 4, d 200-336, 400-640 k 0.88 / 0.98, d 337-660, 0.4-1.8 M 0.80 /
 // 0.97; k = 5, d 280-556 0.80 / 0.95, tiles 0.90 / 0.97; k = 8, d 259-507, 250-400 k 0.93 /
-// 1.05, tiles of exponential series 0.71 / 0.78; one word a digit instead of pairs (no room
-// for them) 0.57 to 0.9 at every k.
+// 1.05, tiles of exponential series 0.71 / 0.78.
 bool mma_takes(int k, int d, const int32_t* supp_ptr, int32_t m0, int32_t m1, bool whole, size_t optin) {
   if (m0 >= m1 || !mma_has(k)) return false;
   if (d < (k == 4 ? 136 : k == 5 ? 256 : k == 8 ? 72 : 56)) return false;
-  if (whole && (mma_smem_bytes(k, d, 1) > optin || !mma_pairs(k, d))) return false;
+  if (whole && mma_smem_bytes(k, d, 1) > optin) return false;
   // products and layers of the monomials (3 n - 3 and n of one of n >= 2 variables)
   int64_t jobs = 0;
   int32_t layers = 1;
@@ -1236,19 +1211,18 @@ bool mma_takes(int k, int d, const int32_t* supp_ptr, int32_t m0, int32_t m1, bo
   return work >= least;
 }
 
-void* mma_kernel(int k, bool tiled, int dmax) {
-  const bool pairs = mma_pairs(k, dmax);
+void* mma_kernel(int k, bool tiled) {
   switch (k) {
-    case 4: return mma_fn<4>(tiled, pairs);
-    case 5: return mma_fn<5>(tiled, pairs);
-    case 8: return mma_fn<8>(tiled, pairs);
-    case 10: return mma_fn<10>(tiled, pairs);
+    case 4: return mma_fn<4>(tiled);
+    case 5: return mma_fn<5>(tiled);
+    case 8: return mma_fn<8>(tiled);
+    case 10: return mma_fn<10>(tiled);
     default: return nullptr;
   }
 }
 
 size_t mma_smem_bytes(int k, int dmax, int depth) {
-  const BufLayout lay = buf_layout(slice_digits(k), mma_stride(k), dmax + 1, dmax + 1, mma_pairs(k, dmax));
+  const BufLayout lay = buf_layout(slice_digits(k), mma_stride(k), dmax + 1, dmax + 1);
   return 4 * (static_cast<size_t>(kMiscWords) + static_cast<size_t>(depth >= 2 ? 2 : 1) * static_cast<size_t>(lay.words));
 }
 
@@ -1270,7 +1244,7 @@ int mma_threads(int k, int dmax) {
 
 size_t mma_tiled_smem_bytes(int k, int tile, int xrows) {
   return 4 * (static_cast<size_t>(kMiscWords) +
-              static_cast<size_t>(buf_layout(slice_digits(k), mma_stride(k), xrows, tile + xrows, true).words));
+              static_cast<size_t>(buf_layout(slice_digits(k), mma_stride(k), xrows, tile + xrows).words));
 }
 
 }  // namespace pes

@@ -249,9 +249,9 @@ extern "C" pes_status pes_eval_grad_static(const int32_t* supp_ptr, const int32_
               " does not fit the shared-memory staging of whole series");
     return PES_EUNSUPPORTED_SIZE;
   }
-  STATIC_CUDA(pes::dag_prepare(k, arith, smem, d));
+  STATIC_CUDA(pes::dag_prepare(k, arith, smem));
   int per_sm = 0;
-  STATIC_CUDA(pes::dag_occupancy(k, arith, threads, smem, d, &per_sm));
+  STATIC_CUDA(pes::dag_occupancy(k, arith, threads, smem, &per_sm));
   if (per_sm < 1) {
     set_error("convolution kernel does not fit on an SM");
     return PES_EUNSUPPORTED_SIZE;

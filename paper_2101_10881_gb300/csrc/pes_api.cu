@@ -334,8 +334,8 @@ struct Exec {
     if (smem > static_cast<size_t>(optin))
       return fail(PES_EUNSUPPORTED_SIZE, "degree " + std::to_string(dmax) + " needs " + std::to_string(smem) +
                                              " bytes of shared memory at k=" + std::to_string(k));
-    PES_CUDA(pes::dag_prepare(k, arith, smem, dmax, tile > 0));
-    PES_CUDA(pes::dag_occupancy(k, arith, threads, smem, dmax, &blocks_per_sm, tile > 0));
+    PES_CUDA(pes::dag_prepare(k, arith, smem, tile > 0));
+    PES_CUDA(pes::dag_occupancy(k, arith, threads, smem, &blocks_per_sm, tile > 0));
     if (blocks_per_sm < 1) return fail(PES_EUNSUPPORTED_SIZE, "convolution kernel does not fit on an SM");
     if (ctas_per_sm > 0) blocks_per_sm = std::min(blocks_per_sm, ctas_per_sm);
     pes_status s = upload(&inst, insts);
@@ -371,9 +371,9 @@ struct Exec {
       return fail(PES_EUNSUPPORTED_SIZE, "fewer lanes than pairs of a tile");
     if (tile == 0 && arith != pes::ARITH_FP64 && L.n > 0 && std::max(1, sp) > L.fparts)
       return fail(PES_EINTERNAL, "parts per job beyond the job flags");
-    PES_CUDA(pes::dag_prepare(k, arith, b, dmax, tile > 0));
+    PES_CUDA(pes::dag_prepare(k, arith, b, tile > 0));
     int bps = 0;
-    PES_CUDA(pes::dag_occupancy(k, arith, t, b, dmax, &bps, tile > 0));
+    PES_CUDA(pes::dag_occupancy(k, arith, t, b, &bps, tile > 0));
     if (bps < 1) return fail(PES_EUNSUPPORTED_SIZE, "configuration does not fit on an SM");
     smem = b;
     depth = dp;
@@ -649,9 +649,9 @@ pes_status tune_launch(Exec& E, JobList& L, const std::string& key, Run run, cud
         for (int32_t t : ts) {
           const size_t b = E.smem_at(dp, t);
           if (b == 0) continue;
-          PES_CUDA(pes::dag_prepare(E.k, E.arith, b, E.dmax, E.tile > 0));
+          PES_CUDA(pes::dag_prepare(E.k, E.arith, b, E.tile > 0));
           int occ = 0;
-          PES_CUDA(pes::dag_occupancy(E.k, E.arith, t, b, E.dmax, &occ, E.tile > 0));
+          PES_CUDA(pes::dag_occupancy(E.k, E.arith, t, b, &occ, E.tile > 0));
           for (int32_t c = std::max(1, occ); c >= std::max(1, occ - 1); --c) {
             pes_status s = E.configure(t, c, dp, sp, L);
             if (s != PES_OK) continue;

@@ -109,3 +109,41 @@ def test_systems_and_batches_have_the_bits_of_single_plans(torch, k):
         pv, pg = pes.Plan(supp, n, dd, k, with_vjp=False, arith="tensor").eval_grad(cuda(torch, c), cuda(torch, z))
         assert torch.equal(bv[vo:vo + pv.numel()], pv.reshape(-1)) and torch.equal(bg[go:go + pg.numel()], pg.reshape(-1))
         vo, go = vo + pv.numel(), go + pg.numel()
+
+
+def against_the_integer_pipe(torch, k, d, supp, n, coeff, inputs):
+    C, Z, U = (cuda(torch, a) for a in (coeff, inputs, inputs[:, 0]))
+    got, infos = [], []
+    for arith in ("tensor", "int"):
+        plan = pes.Plan(supp, n, d, k, arith=arith)
+        got.append([*plan.eval_grad(C, Z), *plan.vjp(C, Z, U, reuse_forward=True)])
+        plan.check()
+        infos.append(plan.info())
+    for a, b in zip(*got):
+        assert normwise_err(a.cpu().numpy(), b.cpu().numpy()) <= close(k)
+    return infos
+
+
+@pytest.mark.parametrize("k,d,tile", [(8, 509, 0), (8, 520, 128), (5, 555, 0), (5, 600, 128), (4, 660, 0), (4, 700, 128),
+                                      (10, 471, 0), (10, 472, 128)])
+def test_whole_series_and_tiles(torch, k, d, tile):
+    """The tiled kernel takes the degrees whose staged pairs do not fit in shared memory, also
+    where 28-bit digits would."""
+    rng = np.random.default_rng(d)
+    info, _ = against_the_integer_pipe(torch, k, d, [[0, 1, 2], [1, 2]], 3, random_md(rng, k, (3, d + 1)),
+                                       random_md(rng, k, (3, d + 1)))
+    assert info["tile"] == tile
+
+
+@pytest.mark.parametrize("k,d", [(10, 152), (10, 700), (10, 1300), (8, 300), (8, 2500), (5, 200), (4, 330), (4, 2500)])
+def test_maximal_slices(torch, k, d):
+    """Every slice of every coefficient near its largest value and of one sign: the
+    accumulators' upper parts are moved as often as ever, and carried in mid-series beyond 563
+    terms at k = 10 and 2339 at k = 8."""
+    from fractions import Fraction
+    W = 10 if k == 10 else 9
+    f = sum(Fraction(2 ** (W - 1) - 1, 2 ** (W * p)) for p in range(1, 53 * k // W + 2))
+    x = np.array(synth.round_fraction_to_limbs(f, k))
+    coeff, inputs = np.zeros((k, 2, d + 1)), np.zeros((k, 2, d + 1))
+    coeff[:] = inputs[:] = x[:, None, None]
+    against_the_integer_pipe(torch, k, d, [[0, 1]], 2, coeff, inputs)
