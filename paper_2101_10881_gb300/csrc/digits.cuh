@@ -57,6 +57,8 @@ constexpr int DIGIT_BITS_INT = 28;
 // grid of a zero coefficient: far below any real grid so that every term with
 // it is skipped
 constexpr int32_t GRID_ZERO = -(1 << 28);
+// series whose grids lie below are taken for zero (2^-2800000 with 28-bit digits)
+constexpr int32_t GRID_LOW = -100000;
 
 // L: smallest number of digits with B (L - 1) >= 53 k + 28 (12 guard bits plus
 // log2 of (1024 terms x 40 digit products)), see the error budget above.

@@ -479,7 +479,7 @@ __global__ void __launch_bounds__(NARROW ? kNarrowThreads : dag_max_threads(K),
         const int32_t g = max(gx[j], gy[j]);
         int32_t o[L];
         int32_t gz = GRID_ZERO;
-        if (g < -100000) {
+        if (g < GRID_LOW) {
 #pragma unroll
           for (int p = 0; p < L; ++p) o[p] = 0;
         } else {
@@ -690,7 +690,7 @@ __global__ void __launch_bounds__(NARROW ? kNarrowThreads : dag_max_threads(K),
         const int32_t g = gs[j];
         int32_t o[L];
         int32_t gz = GRID_ZERO;
-        if (g < -100000) {
+        if (g < GRID_LOW) {
   #pragma unroll
           for (int p = 0; p < L; ++p) o[p] = 0;
         } else {
@@ -920,7 +920,7 @@ __global__ void __launch_bounds__(dag_max_threads(K), INTV ? dag_min_ctas(K) : 1
           const int32_t g = max(gx[t], gy[t]);
           int32_t o[L];
           int32_t gz = GRID_ZERO;
-          if (g < -100000) {
+          if (g < GRID_LOW) {
 #pragma unroll
             for (int p = 0; p < L; ++p) o[p] = 0;
           } else {
@@ -1089,7 +1089,7 @@ __global__ void __launch_bounds__(dag_max_threads(K), INTV ? dag_min_ctas(K) : 1
           const int32_t g = gs[t];
           int32_t o[L];
           int32_t gz = GRID_ZERO;
-          if (g < -100000) {
+          if (g < GRID_LOW) {
 #pragma unroll
             for (int p = 0; p < L; ++p) o[p] = 0;
           } else {
@@ -1126,6 +1126,7 @@ struct Fmt {
   static constexpr int B = MMA ? 2 * W : AR == ARITH_INT ? DIGIT_BITS_INT : DIGIT_BITS;
   static constexpr int L = MMA ? slice_digits(K) : digits_for_k(K, B);
   static constexpr int RW = MMA ? L : row_words(L, AR == ARITH_INT);
+  static constexpr int32_t LOW = MMA ? slice_grid_low(K) : GRID_LOW;  // grids below: zero
   // words a sum of series is formed in, digit position 0 the top of its largest grid
   static constexpr int NW = MMA ? sum_words(K) : L;
 
@@ -1201,7 +1202,7 @@ __global__ void __launch_bounds__(256) unpack_kernel(CopyArgs a) {
   const int32_t* grids = rows + static_cast<long long>(in.S) * RW;
   for (int j = lane; j <= in.d; j += 32) {
     const int32_t g = F::grid(grids[j]);
-    if (g < -100000) {
+    if (g < F::LOW) {
 #pragma unroll
       for (int l = 0; l < K; ++l) dst[l * r.lstride + j] = 0.0;
       continue;
@@ -1284,7 +1285,7 @@ __device__ __forceinline__ void add_sums(const AddArgs& a, long long items, long
   int32_t gmax = 2 * GRID_ZERO;
   if (a.mode == 2) {
     gmax = valid ? a.grid_io[item] : gmax;
-    if (F::MMA && gmax >= -100000) gmax = sum_anchor<B>(gmax);
+    if (F::MMA) gmax = gmax >= GRID_LOW ? sum_anchor<B>(gmax) : 2 * GRID_ZERO;
   } else {
     if (valid) {
 #pragma unroll 4
@@ -1299,7 +1300,7 @@ __device__ __forceinline__ void add_sums(const AddArgs& a, long long items, long
       for (int t = 0; t < gw; ++t) gmax = max(gmax, gm_s[warp - sw + t]);
     }
     if (a.mode == 1) {
-      if (valid && gl == 0) a.grid_io[item] = F::MMA && gmax >= -100000 ? sum_grid28<B>(gmax) : gmax;
+      if (valid && gl == 0) a.grid_io[item] = F::MMA && gmax >= F::LOW ? sum_grid28<B>(gmax) : gmax;
       return;
     }
   }
@@ -1307,7 +1308,7 @@ __device__ __forceinline__ void add_sums(const AddArgs& a, long long items, long
   int last = NW - 1, f = 0;  // tensor cores: where the sum ends
   if constexpr (F::MMA) {
     int32_t floor28 = 0;
-    if (gmax >= -100000) sum_end<K, B>(gmax, a.mode == 2 ? a.grid_io[item] : sum_grid28<B>(gmax), last, f, floor28);
+    if (gmax >= F::LOW) sum_end<K, B>(gmax, a.mode == 2 ? a.grid_io[item] : sum_grid28<B>(gmax), last, f, floor28);
   }
 
   // every lane sums its contributions' digits, shifted to the common grid
@@ -1324,7 +1325,7 @@ __device__ __forceinline__ void add_sums(const AddArgs& a, long long items, long
       int32_t half[NW];
 #pragma unroll
       for (int p = 0; p < NW; ++p) half[p] = 0;
-      if (valid && gmax >= -100000) {
+      if (valid && gmax >= F::LOW) {
 #pragma unroll 2
         for (int c = ao.cbeg + gl; c < ao.cend; c += G) {
           const int32_t* slot = base + static_cast<long long>(a.contrib[c]) * in.ws_sstride;
@@ -1358,7 +1359,7 @@ __device__ __forceinline__ void add_sums(const AddArgs& a, long long items, long
   if (!summed) {
 #pragma unroll
     for (int p = 0; p < NW; ++p) acc[p] = 0;
-    if (valid && gmax >= -100000) {
+    if (valid && gmax >= F::LOW) {
 #pragma unroll 2
       for (int c = ao.cbeg + gl; c < ao.cend; c += G) {
         const int32_t* slot = base + static_cast<long long>(a.contrib[c]) * in.ws_sstride;
@@ -1419,7 +1420,7 @@ __device__ __forceinline__ void add_round(const AddArgs& a, long long w, const l
       long long out[L28];
 #pragma unroll
       for (int p = 0; p < L28; ++p) out[p] = 0;
-      if (gmax >= -100000) {
+      if (gmax >= F::LOW) {
         int last, f;
         int32_t floor28;
         sum_end<K, B>(gmax, a.grid_io[item], last, f, floor28);
@@ -1453,8 +1454,8 @@ __device__ __forceinline__ void add_round(const AddArgs& a, long long w, const l
   if (a.to_ws) {
     int32_t* slot = a.ws + in.ws_base + ao.dst_off * in.ws_sstride;
     int32_t dg[NW];  // the first L digits are kept
-    const int32_t gz = gmax < -100000 ? GRID_ZERO : sum_to_digits<NW, B>(E, gmax + 1, dg);
-    if (gmax < -100000) {
+    const int32_t gz = gmax < F::LOW ? GRID_ZERO : sum_to_digits<NW, B>(E, gmax + 1, dg);
+    if (gmax < F::LOW) {
 #pragma unroll
       for (int p = 0; p < NW; ++p) dg[p] = 0;
     }
@@ -1462,7 +1463,7 @@ __device__ __forceinline__ void add_round(const AddArgs& a, long long w, const l
     return;
   }
   double* dst = a.dst[ao.dst_sel] + ao.dst_off + j * ao.dst_jstride;
-  if (gmax < -100000) {
+  if (gmax < F::LOW) {
 #pragma unroll
     for (int l = 0; l < K; ++l) dst[l * ao.dst_lstride] = 0.0;
     return;
@@ -1517,7 +1518,7 @@ __host__ __device__ void round_sum_item(const RoundArgs& a, long long item) {
   double* dst = o == 0 ? a.value + j : a.grad + (o - 1) * D1 + j;
   const long long ls = o == 0 ? D1 : static_cast<long long>(a.n) * D1;
   const int32_t g = a.grids[item];
-  if (g < -100000) {
+  if (g < GRID_LOW) {
     for (int l = 0; l < K; ++l) dst[l * ls] = 0.0;
     return;
   }

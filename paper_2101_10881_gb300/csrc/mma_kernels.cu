@@ -427,6 +427,7 @@ struct Group {
   static constexpr float kUnit = 281474976710656.f;    // 2^48: one slice product
   static constexpr float kUnitHi = 549755813888.f;     // 2^39: the unit of the upper parts, 2^9 products
   static constexpr float kSplit = 1.5f / 65536.f;      // 1.5 2^23 units of the upper parts
+  static constexpr int kLow = 4 * slice_grid_low(K);   // sums of grids below: zero
   float acc[NT][NB][4];  // rows 2 g - 1 (elements 0, 1: columns 2 tl, 2 tl + 1) and 2 g (2, 3) of each block
   float up[NT][NB][4];   // the upper parts
   int gs[NT];            // four times the reference grid of column g of each tile
@@ -463,14 +464,14 @@ struct Group {
     int lo = 1 << 30, hi = -(1 << 30);
 #pragma unroll
     for (int t = 0; t < NT; ++t) {
-      const bool some = gm[t] >= -400000;
+      const bool some = gm[t] >= kLow;
       lo = min(lo, some ? gm[t] : lo);
       hi = max(hi, some ? gm[t] : hi);
     }
     gs_lo = __reduce_min_sync(0xffffffffu, lo);
     gs_hi = __reduce_max_sync(0xffffffffu, hi);
 #pragma unroll
-    for (int t = 0; t < NT; ++t) gs[t] = gm[t] >= -400000 ? gm[t] : max(gs_hi, -400000);
+    for (int t = 0; t < NT; ++t) gs[t] = gm[t] >= kLow ? gm[t] : max(gs_hi, kLow);
   }
 
   // the Toeplitz fragments of the row at xr: word offset 4 (kap - 1), slice rho
@@ -603,7 +604,7 @@ struct Group {
     // terms from `from` on take the flat loop
     const int lo = gs_hi - a.gmax - 4 * PZ, hi = gs_lo - a.gmax + 4 * M::RA;
     int from = n[0];
-    if (a.flat && gs_hi >= -400000 && lo <= hi) {
+    if (a.flat && gs_hi >= kLow && lo <= hi) {
       from = 0;
       for (int u = threadIdx.x & 31; u < n[0]; u += 32) {
         const int gx = static_cast<int>(lds(a.ga + 4 * u));
@@ -760,7 +761,7 @@ __device__ __forceinline__ void add_rows(const int32_t* xs, const int32_t* ys, i
   const int32_t g = max(gx, gy);
   int32_t o[L];
   int32_t gz = GRID_ZERO;
-  if (g < -100000) {
+  if (g < slice_grid_low(K)) {
 #pragma unroll
     for (int p = 0; p < L; ++p) o[p] = 0;
   } else {

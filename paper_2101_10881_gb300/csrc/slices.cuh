@@ -33,6 +33,9 @@ PES_HDC int slice_digits(int k) {
   return (DIGIT_BITS_INT * (digits_for_k(k, DIGIT_BITS_INT) - 1) + slice_digit_bits(k) - 1) / slice_digit_bits(k) + 1;
 }
 
+// Grids below are taken for zero: the line of the 28-bit digits, 2^-2800000.
+PES_HDC int32_t slice_grid_low(int k) { return -(-GRID_LOW * DIGIT_BITS_INT / slice_digit_bits(k)); }
+
 // word of a balanced digit v, |v| <= 2^(2W-1)
 template <int W>
 PES_HD uint32_t slice_encode(int32_t v) {

@@ -147,3 +147,23 @@ def test_maximal_slices(torch, k, d):
     coeff, inputs = np.zeros((k, 2, d + 1)), np.zeros((k, 2, d + 1))
     coeff[:] = inputs[:] = x[:, None, None]
     against_the_integer_pipe(torch, k, d, [[0, 1]], 2, coeff, inputs)
+
+
+@pytest.mark.parametrize("k", KT)
+def test_products_far_below_the_smallest_double(torch, k):
+    """Running products down to 2^-1900000 come back to 1: series are taken for zero below
+    2^-2800000 only, as on the integer pipe."""
+    n, d = 3800, 1
+    inputs = np.zeros((k, n, d + 1))
+    inputs[0, :, 0] = np.where(np.arange(n) < n // 2, 2.0 ** -1000, 2.0 ** 1000)
+    inputs[0, :, 1] = inputs[0, :, 0] * (1 + np.arange(n) % 7)
+    coeff = np.zeros((k, 2, d + 1))
+    coeff[0, 1, 0] = 1.0
+    got = []
+    for arith in ("tensor", "int"):
+        plan = pes.Plan([list(range(n))], n, d, k, with_vjp=False, arith=arith)
+        got.append([t.cpu().numpy() for t in plan.eval_grad(cuda(torch, coeff), cuda(torch, inputs))])
+        plan.check()
+    assert got[0][0][0, 0] == 1.0
+    for a, b in zip(*got):
+        assert normwise_err(a, b) <= close(k)
