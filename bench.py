@@ -142,6 +142,27 @@ def digit_fma_flops(conv_jobs, d, digits):
     return conv_jobs * (d + 1) * (d + 2) // 2 * (L * (L + 1) // 2) * 2
 
 
+# f16 mma.sync m16n8k16 with fp32 sums: 301 T multiply-adds/s on a loop of independent products of this GPU
+MMA_TFLOPS = 602.0
+
+
+def slice_product_flops(conv_jobs, d, k, digits):
+    """Flops (2 per multiply-add) of the slice products the tensor-core kernels
+    issue: per term of an 8-column tile b (b + 1) / 2 products of 16 x 16 x 8
+    for the b 16-slice blocks of a coefficient (blocks above the diagonal are
+    not issued, columns past a tile's edge are)."""
+    bits = 20 if k >= 10 else 18
+    slices = 2 * (-(-28 * (digits - 1) // bits) + 1)
+    blocks = -(-slices // 16)
+    terms = sum(d + 1 - 8 * t for t in range((d + 8) // 8))
+    return conv_jobs * terms * (blocks * (blocks + 1) // 2) * 2048 * 2
+
+
+def int_frac(plan, macs, ms, peak):
+    """Share of the integer pipe's peak of a plan that runs there, else None."""
+    return macs / (ms * 1e-3) / 1e12 / peak if peak and plan.arith() == "int" else None
+
+
 # ---------------------------------------------------------------------------
 # clocks during the timed region
 # ---------------------------------------------------------------------------
@@ -342,7 +363,7 @@ def kernel_source_hash():
     same."""
     import re
     h = hashlib.sha256()
-    for f in ("kernels.cu", "digits.cuh", "kernels.hpp", "mma_kernels.cu", "slices.cuh"):
+    for f in ("kernels.cu", "digits.cuh", "kernels.hpp", "dag_sync.cuh", "mma_kernels.cu", "slices.cuh"):
         path = os.path.join(ROOT, "paper_2101_10881_gb300", "csrc", f)
         if not os.path.exists(path):
             continue
@@ -478,22 +499,29 @@ def ours_arm(args, world, rank, local):
     mean_conv = statistics.mean(conv_ms)
     work = (f"{info['conv_jobs']} convolutions x {(prob.d + 1) * (prob.d + 2) // 2} terms x "
             f"{info['digits'] * (info['digits'] + 1) // 2} digit products")
-    arith = info["arith_name"]
+    arith = plan.arith()
     nsm = torch.cuda.get_device_properties(dev).multi_processor_count
     clk_max_mhz = clk.get("sm_max_mhz")
+    derived = 8 * 4 * nsm * clk_max_mhz * 1e6 / 1e12 if clk_max_mhz else None
+    int_unit = derived if derived else int_peak
     if arith == "fp64":
         achieved = digit_flops / (mean_conv * 1e-3) / 1e12
         roofline = {"bound": "alu", "pipe": "fp64 (DFMA)", "achieved": achieved, "peak": fp64_peak,
                     "unit": "TFLOP/s", "frac": achieved / fp64_peak,
                     "peak_source": "measured: pes_fp64_peak DFMA microbenchmark (burst, all SMs), this run"}
+    elif arith == "tensor":
+        flops = slice_product_flops(info["conv_jobs"], prob.d, prob.k, info["digits"])
+        achieved = flops / (mean_conv * 1e-3) / 1e12
+        work = f"{info['conv_jobs']} convolutions, {flops // 2 // info['conv_jobs']} slice multiply-adds each"
+        roofline = {"bound": "tensor", "pipe": "tensor (f16 mma.sync m16n8k16 of 10-bit slices, exact fp32 sums)"
+                    if prob.k >= 10 else "tensor (f16 mma.sync m16n8k16 of 9-bit slices, exact fp32 sums)",
+                    "achieved": achieved, "peak": MMA_TFLOPS, "unit": "TFLOP/s", "frac": achieved / MMA_TFLOPS,
+                    "peak_source": "measured once: mma.sync m16n8k16 f16 -> fp32, a loop of independent products, all "
+                                   "SMs (tcgen05, which cuBLAS takes, has about three times this rate)"}
     else:
         achieved = digit_flops / 2 / (mean_conv * 1e-3) / 1e12
-        derived = 8 * 4 * nsm * clk_max_mhz * 1e6 / 1e12 if clk_max_mhz else None
-        peak = derived if derived else int_peak
-        roofline = {"bound": "alu", "pipe": "int (IMAD.WIDE 32x32+64)",
-                    "note": "the 28-bit digit products of the integer pipe, in the time the plan took: wide tables "
-                            "form theirs on the tensor cores (f16 mma.sync), where this exceeds the pipe",
-                    "achieved": achieved, "peak": peak,
+        peak = int_unit
+        roofline = {"bound": "alu", "pipe": "int (IMAD.WIDE 32x32+64)", "achieved": achieved, "peak": peak,
                     "unit": "Tops/s", "frac": achieved / peak,
                     "peak_source": ("derived: 8 lanes/clock per SM sub-partition (a 32x32+64 multiply-add "
                                     "occupies the heavy FMA pipe 4 clocks per warp, ncu) x 4 x SMs x max SM clock"
@@ -506,7 +534,7 @@ def ours_arm(args, world, rank, local):
     # ---- the other multiply-accumulate pipe, kernel-only, same workload ----
     variants = {arith: {"ms_per_step": total_ms / args.steps, "value": value, "roofline_frac": roofline["frac"],
                         "pipe": roofline["pipe"], "digits": info["digits"]}}
-    if not args.no_variants and arith == "int":
+    if not args.no_variants and arith != "fp64":
         p64 = pes.Plan(prob.supports, prob.n, prob.d, prob.k, arith="fp64", with_vjp=False, profile=True)
         i64 = p64.info()
         sms, cms, _ = timed(p64, max(2, min(args.steps, 3)))
@@ -520,7 +548,7 @@ def ours_arm(args, world, rank, local):
     out = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": total_ms / args.steps, "higher_is_better": True,
-        "scaling": "weak", "vs_baseline": None, "dtype": "int64" if arith == "int" else "f64",
+        "scaling": "weak", "vs_baseline": None, "dtype": "f64" if arith == "fp64" else "int64",
         "data": "synthetic", "config": dict(workload_config(prob, args), arith_used=arith,
                                             values="k-double series (k float64 limbs per coefficient)"),
         "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,
@@ -548,24 +576,23 @@ def ours_arm(args, world, rank, local):
     if not args.no_autograd:
         out["autograd"] = autograd_measure(args, dev, flush)
     if args.workload == "p2" and not args.no_powers:
-        out["powers"] = powers_measure(args, dev, flush, roofline["peak"] if arith == "int" else None)
+        out["powers"] = powers_measure(args, dev, flush, int_unit)
     if args.workload == "p2" and not args.no_complex:
-        out["complex"] = complex_measure(args, dev, flush, roofline["peak"] if arith == "int" else None)
+        out["complex"] = complex_measure(args, dev, flush, int_unit)
     if args.workload == "p2" and not args.no_large_degree:
-        out["large_degree"] = large_degree_measure(args, dev, flush, roofline["peak"] if arith == "int" else None)
+        out["large_degree"] = large_degree_measure(args, dev, flush, int_unit)
     if args.workload == "p2" and not args.no_system:
-        out["system"] = system_measure(args, dev, flush, roofline["peak"] if arith == "int" else None)
+        out["system"] = system_measure(args, dev, flush, int_unit)
     if world > 1 and args.shard:
         out["shard"] = shard_measure(args, dev, world, rank, prob, ops_step, flush)
-    int_peak_unit = roofline["peak"] if arith == "int" else None
     if args.workload == "p2" and not args.no_config0:
         out["config0"] = config0_measure(args, dev, flush)
     if args.workload == "p2" and not args.no_config4:
         out["config4"] = config4_measure(args, dev)
     count = 2048 if args.batch_count is None else args.batch_count
     if count > 0:
-        out["batched"] = batch_measure(args, dev, count, k=2, peak=int_peak_unit)
-        out["batched_k8"] = batch_measure(args, dev, min(count, 512), k=8, peak=int_peak_unit)
+        out["batched"] = batch_measure(args, dev, count, k=2, peak=int_unit)
+        out["batched_k8"] = batch_measure(args, dev, min(count, 512), k=8, peak=int_unit)
         out["batched_small"] = batch_measure(args, dev, 2048, small=True)
     if rank == 0 and world == 1 and not args.no_cpu_baseline:
         sub = cpu_sample(prob, args.cpu_sample_vars)
@@ -773,8 +800,8 @@ def powers_measure(args, dev, flush, peak):
     return {"workload": "p2-like, n=128, 128 monomials of 64 variables, exponents uniform in 1-3, d=152, k=10",
             "ms_per_step": ms, "value": ops / (ms * 1e-3) / 1e12, "unit": UNIT,
             "conv_jobs": info["conv_jobs"], "power_and_factor_jobs": info["conv_jobs"] - plain,
-            "roofline_frac": (macs / (cms * 1e-3) / 1e12) / peak if peak else None,
-            "kernel_ms": cms, "threads_per_cta": info["threads"], "arith": info["arith_name"]}
+            "roofline_frac": int_frac(plan, macs, cms, peak),
+            "kernel_ms": cms, "threads_per_cta": info["threads"], "arith": plan.arith()}
 
 
 def complex_measure(args, dev, flush, peak):
@@ -831,8 +858,8 @@ def complex_measure(args, dev, flush, peak):
     return {"workload": "p2-like, n=128, 128 monomials of 64 variables, complex series, d=152, k=10",
             "ms_per_step": ms, "value": ops / (ms * 1e-3) / 1e12, "unit": UNIT,
             "real_convolutions": products, "series_additions": series_adds,
-            "roofline_frac": (macs / (cms * 1e-3) / 1e12) / peak if peak else None,
-            "kernel_ms": cms, "threads_per_cta": info["threads"], "arith": info["arith_name"],
+            "roofline_frac": int_frac(plan, macs, cms, peak),
+            "kernel_ms": cms, "threads_per_cta": info["threads"], "arith": plan.arith(),
             "workspace_bytes": info["workspace_bytes"],
             "vjp_ms": statistics.mean(vjp_ms), "vjp_over_forward": statistics.mean(vjp_ms) / ms}
 
@@ -911,7 +938,7 @@ def system_measure(args, dev, flush, peak):
             "ms_per_step": res["system"], "value": ops / (res["system"] * 1e-3) / 1e12, "unit": UNIT,
             "plans_ms_per_step": res["plans"], "plans_over_system": res["plans"] / res["system"],
             "conv_jobs": info["conv_jobs"], "jacobian_layout": "matrix [k][d+1][P][n]",
-            "roofline_frac": (macs / (conv_ms * 1e-3) / 1e12) / peak if peak else None,
+            "roofline_frac": int_frac(sysp, macs, conv_ms, peak),
             "kernel_ms": conv_ms, "workspace_bytes": info["workspace_bytes"],
             "system_equals_plans_bitwise": bool(same), "launches_system": 3, "launches_plans": 3 * len(plans),
             "autograd": {"forward_ms": statistics.mean(t[0] for t in fb),
@@ -957,8 +984,8 @@ def large_degree_measure(args, dev, flush, peak):
         macs = digit_fma_flops(info["conv_jobs"], d, info["digits"]) / 2
         out[name] = {"d": d, "tile": info["tile"], "ms_per_step": ms, "value": ops / (ms * 1e-3) / 1e12,
                      "unit": UNIT, "kernel_ms": cms,
-                     "roofline_frac": (macs / (cms * 1e-3) / 1e12) / peak if peak else None,
-                     "threads_per_cta": info["threads"], "grid": info["grid"],
+                     "roofline_frac": int_frac(plan, macs, cms, peak),
+                     "arith": plan.arith(), "threads_per_cta": info["threads"], "grid": info["grid"],
                      "workspace_bytes": info["workspace_bytes"]}
         del plan, C, Z
     out["workload"] = "p2-like, n=128, 128 monomials of 64 variables, k=10, random series"
@@ -1044,7 +1071,8 @@ def batch_measure(args, dev, count, small=False, k=None, peak=None):
                     "plain_frac_of_int_peak": at_peak_ms / res["plain"],
                     "ceiling_plain_over_batched": res["plain"] / at_peak_ms,
                     "ceiling_rule": "plain time over the time of the batch's digit multiply-adds at the integer "
-                                    "pipe's unit-count peak (no batched launch can be faster)"})
+                                    "pipe's unit-count peak: no batched launch on the integer pipe can be faster "
+                                    "(instances on the tensor cores can)"})
     return out
 
 
@@ -1160,13 +1188,14 @@ def sweep_arm(args, world, rank):
                 e2.synchronize()
                 sfb.append((e0.elapsed_time(e1), e1.elapsed_time(e2)))
             sysp.check()
+            sys_arith = sysp.arith()
             del sysp, Csys, sv, sj, v_sys, Zs, Cq
             ops = dp_equiv_ops(conv_jobs, add_jobs, d, k)
             row = {"cell": f"k={k} d={d}", "k": k, "d": d, "forward_ms": fwd, "backward_ms": bwd,
                    "backward_over_forward": bwd / fwd if fwd > 0 else None,
                    "forward_dp_equiv_tflops": ops / (fwd * 1e-3) / 1e12, "conv_jobs": conv_jobs,
                    "closed_form_err": max(errs), "tol": tol[k], "within_tol": max(errs) <= tol[k],
-                   "arith": info[0]["arith_name"], "system_values_and_jacobian_ms": min(st),
+                   "arith": sys_arith, "system_values_and_jacobian_ms": min(st),
                    "system_values_equal_plans_bitwise": bool(sys_same),
                    "system_forward_ms": min(t[0] for t in sfb), "system_backward_ms": min(t[1] for t in sfb)}
             rows.append(row)
