@@ -62,7 +62,7 @@ typedef struct pes_batch_s* pes_batch_t;
  * digits of 18 or 20 bits; its outputs differ from PES_ARITH_INT's below the last limb.
  * PES_ARITH_AUTO takes the integer pipe, or the tensor cores for polynomials with many
  * products a layer: at k = 10 and 8 from degrees 56 and 72 on, at k = 4 from 136 on, at
- * k = 5 between 256 and 279.  The choice depends on the
+ * k = 5 between 256 and 277.  The choice depends on the
  * sizes of the monomials, k and d (pes_auto_arith tells it): all plans of one polynomial
  * make the same, but for one (or a batch) whose series, up to 1.54 times as long on the
  * tensor cores, do not fit the device memory: it takes the integer pipe.  Plans given one
@@ -74,7 +74,9 @@ typedef struct {
   int32_t threads;     /* threads per CTA of the convolution kernel (a multiple of 32), 0 = automatic.
                           Integer pipe: the lanes are spread evenly over the coefficient pairs (j, d-j),
                           automatic = two lanes per pair (one per output coefficient; three at k = 10),
-                          at least one lane per pair; FP64 pipe: automatic = 128 */
+                          at least one lane per pair; FP64 pipe: automatic = 128; tensor cores: automatic =
+                          as many warps as fill the registers with the CTAs that fit an SM, at most one per
+                          8 coefficients */
   int32_t ctas_per_sm; /* persistent CTAs per SM; 0 = as many as fit */
   int32_t with_vjp;    /* 1: also build the tables of pes_vjp (default 1) */
   int64_t timeout_ms;  /* bound on every device-side wait; 0 = default (60000) */
@@ -88,18 +90,20 @@ typedef struct {
                           job's operands are complete, stages them while rounding the current one
                           (a separate staging buffer: more shared memory); 0 = automatic (1, and both
                           are tried when autotuning) */
-  int32_t split;       /* parts per convolution job (integer pipe): 1, 2, 4, 8 or 16; each part computes
-                          the output coefficients of a contiguous range of coefficient pairs (j, d-j), so a
-                          job's dependants wait for all its parts; more parts shorten the chains of long
+  int32_t split;       /* parts per convolution job (integer pipe, tensor cores): 1, 2, 4, 8 or 16; each
+                          part computes the output coefficients of a contiguous range of coefficient
+                          pairs (j, d-j), so a job's dependants wait for all its parts; more parts shorten the chains of long
                           monomials; 0 = automatic: the parts double while the table's average layer, times
                           the parts, holds fewer jobs than the launch has CTAs and every part keeps at
                           least 8 coefficient pairs (the p2-like workload at d=152, k=10: 1 for its 128
-                          monomials, 2 for 64 of them, 4 for 32, 8 for 16 or fewer; p3: 1); when
+                          monomials, 2 for 64 of them, 4 for 32, 8 for 16 or fewer; p3: 1; tensor cores:
+                          while all parts of a layer run at once and every part keeps 8 coefficients); when
                           autotuning, 1, 2 and the automatic choice, half and twice it, are tried */
   int32_t tile;        /* 0 = automatic: the whole series of a job's operands are staged in shared memory
                           when they fit (integer / FP64 pipe: d <= 471 / 359 at k=10, 543 / 447 at k=8,
                           839 / 607 at k=5, 991 / 815 at k=4, 1075 / 919 at k=3, 1351 / 1231 at k=2,
-                          1535 / 1487 at k=1), else the tiled kernel with tiles of 128 coefficients.
+                          1535 / 1487 at k=1; tensor cores: the integer pipe's, and d <= 513 at k=8, 563 at
+                          k=5, 669 at k=4), else the tiled kernel with tiles of 128 coefficients.
                           > 0 (a multiple of 8 in [16, 1024]): always the tiled kernel with tiles of this
                           many coefficients: every job is split into output tiles, each accumulated tile
                           pair by tile pair from staged tiles of its operands (any degree up to 16383; the
@@ -161,7 +165,8 @@ pes_status pes_plan_complex(const int32_t* supp_ptr, const int32_t* supp_idx, co
  * the input series and one job table; the products of every monomial are the
  * ones its own plan would compute, so every output is bit-identical to a plan
  * of that polynomial alone in the same arithmetic (pes_get_plan_arith: PES_ARITH_AUTO takes
- * the tensor cores for a system when it would for each of its polynomials).  Evaluate with pes_eval_system (pes_eval_grad is
+ * the tensor cores for a system when it would for each of its polynomials).
+ * Evaluate with pes_eval_system (pes_eval_grad is
  * pes_eval_system with PES_LAYOUT_SERIES); pes_vjp takes one upstream series
  * per polynomial.
  *   P >= 1, poly_ptr: P+1 non-decreasing entries, poly_ptr[0] == 0.
@@ -289,8 +294,8 @@ pes_status pes_get_plan_arith(pes_plan_t plan, int32_t* arith);
  * every rank obtains the value and gradient that one plan of the whole polynomial
  * computes, bit for bit, if all of them are given the same arithmetic
  * (that of the whole polynomial, pes_auto_arith; PES_ARITH_AUTO goes by the monomials of
- * each plan, and differs below the last limb's rounding): the addition stage sums the contributions of every
- * output coefficient on the largest grid among them and rounds once, and both
+ * each plan, and differs below the last limb's rounding): the addition stage sums
+ * the contributions of every output coefficient on the largest grid among them and rounds once, and both
  * the maximum and the sum of integers are exact in any order.  (A sum of the
  * ranks' rounded k-double limbs in floating point would not be.)
  *
@@ -482,18 +487,19 @@ pes_status pes_selftest_timeout(int64_t timeout_ms, int32_t* device_status);
  * and pes_eval_grad (caller-owned device buffers coeff, input, value, grad;
  * asynchronous on `stream`); the outputs are bit for bit those of pes_plan +
  * pes_eval_grad, or, where a plan would take the tensor cores but their longer
- * series exceed the array, of a plan given PES_ARITH_INT.  The job tables are compiled on the host at every call and
- * copied into the array with cudaMemcpyAsync; nothing calls cudaMalloc,
- * cudaFree or an allocating library routine.  Limits, each rejected with
- * PES_EUNSUPPORTED_SIZE (message in pes_last_error):
+ * series exceed the array, of a plan given PES_ARITH_INT.  The job tables are
+ * compiled on the host at every call and copied into the array with
+ * cudaMemcpyAsync; nothing calls cudaMalloc, cudaFree or an allocating library
+ * routine.  Limits, each rejected with PES_EUNSUPPORTED_SIZE (message in
+ * pes_last_error):
  *   - d <= 1023, and the whole operand series of a job must fit one CTA's
  *     shared memory (there is no tiled kernel here): d <= 471 at k=10, 543 at
  *     k=8, 839 at k=5, 991 at k=4;
  *   - tables and workspace within the 64 MiB (of the integer pipe's form): at
  *     d=152, k=10 a series takes 18,560 bytes of workspace (160 rows of 29 words;
  *     19,200 on the tensor cores), so about 3,600 series fit (3,400, and the
- *     integer pipe's form from there on); the workspace holds 3 n_m - 2 series per monomial of n_m >= 2
- *     variables, a_0 and the n inputs.
+ *     integer pipe's form from there on); the workspace holds 3 n_m - 2 series
+ *     per monomial of n_m >= 2 variables, a_0 and the n inputs.
  * Negative d or a NULL buffer is PES_EINVAL, k outside the set
  * PES_EUNSUPPORTED_K.
  *

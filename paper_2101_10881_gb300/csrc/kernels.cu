@@ -1159,9 +1159,11 @@ struct Fmt {
   }
 };
 
-// pack: one warp per series; every lane converts coefficients j = lane, lane+32,
-// ... of the caller's k-limb series into L balanced digits on the grid of the
-// leading limb and writes the digit row and grid into the workspace slot.
+// pack: a warp per series, or per series and share of its coefficients (blockIdx.y);
+// every lane converts coefficients j = lane, lane + 32 gridDim.y, ... of the caller's
+// k-limb series into L balanced digits on the grid of the leading limb and writes the
+// digit row and grid into the workspace slot.  The first thread of a call's first pack
+// launch starts the call: the next epoch, job counters at zero.
 template <int K, int AR>
 __global__ void __launch_bounds__(256) pack_kernel(CopyArgs a) {
   using F = Fmt<K, AR>;
@@ -1758,7 +1760,7 @@ cudaError_t launch_pack(const CopyArgs& a, int k, int arith, cudaStream_t st) {
   // warp went through d / 32 times (66 series, d = 152: 45 -> 17 us; 41 series, d = 1023:
   // 341 -> 30 us).
   const unsigned chunks = static_cast<unsigned>(a.dmax / 32 + 1);
-  const dim3 grid(blocks, std::max(1u, std::min(chunks, 304u / blocks)));
+  const dim3 grid(blocks, std::max(1u, std::min(chunks, 2u * kSms / blocks)));
   PES_DISPATCH_K_ARITH(pack_kernel, k, arith, grid, warps * 32, st, a);
   return cudaGetLastError();
 }
@@ -1776,7 +1778,7 @@ cudaError_t launch_unpack(const CopyArgs& a, int k, int arith, cudaStream_t st) 
 static unsigned add_blocks(AddArgs& a, int64_t items) {
   const int64_t per = 8 / a.group_warps;
   const int64_t sums = (items + per - 1) / per;
-  a.rounds = static_cast<int32_t>(std::max<int64_t>(1, std::min<int64_t>(kAddItems / per, sums / (6 * 152))));
+  a.rounds = static_cast<int32_t>(std::max<int64_t>(1, std::min<int64_t>(kAddItems / per, sums / (6 * kSms))));
   return static_cast<unsigned>((sums + a.rounds - 1) / a.rounds);
 }
 

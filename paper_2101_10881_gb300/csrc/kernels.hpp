@@ -124,7 +124,8 @@ __host__ __device__ constexpr int mma_max_threads(int k) { return k >= 8 ? 384 :
 // series.  mma_kernels.cu holds the rule's line and its times.
 bool mma_takes(int k, int d, const int32_t* supp_ptr, int32_t m0, int32_t m1, bool whole, size_t optin);
 // Column tiles (8 coefficients) a warp of the tensor-core kernels accumulates at once.
-__host__ __device__ constexpr int mma_group_tiles(int k) { return 3; }
+constexpr int kMmaGroupTiles = 3;
+constexpr int kSms = 152;  // SMs of a GB300, for the grids of the packing and addition launches
 constexpr int kMaxSplit = 16;  // largest number of parts a convolution job is split into
 
 // Shared-memory footprint of the DAG kernel for (k, arith, smax, dmax) at

@@ -40,9 +40,9 @@
 //
 // Measured (one GB300, convolution kernel): p2-like d = 152, k = 10, 9.28 ms in the integer
 // pipe's best shape and 10.1 ms in its default one, 5.8 ms here; all pairs of 48 variables
-// with every third a triple, d = 152, k = 4 / 5 / 8 / 10: 0.72 / 0.95 / 2.18 / 2.27 ms ->
-// 0.49 / 0.72 / 1.04 / 1.17 ms, with exponential series 0.55 / 0.70 / 1.57 / 1.72 ->
-// 0.53 / 0.70 / 1.17 / 1.35.
+// with every third a triple, d = 152, k = 4 / 5 / 8 / 10: 0.57 / 0.73 / 1.74 / 1.75 ms ->
+// 0.39 / 0.62 / 0.83 / 0.95 ms, with exponential series 0.54 / 0.70 / 1.69 / 1.74 ->
+// 0.37 / 0.56 / 0.99 / 1.12.
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -112,7 +112,7 @@ struct Mma {
   static constexpr int PZ = SW - L - SP;
   static constexpr int RA = SW - 8 * KS < 4 ? SW - 8 * KS : 4;
   static constexpr int PS = L + kPairLead;        // pairs of a Toeplitz row
-  static constexpr int NT = mma_group_tiles(K);   // column tiles of 8 coefficients a warp accumulates at once
+  static constexpr int NT = kMmaGroupTiles;       // column tiles of 8 coefficients a warp accumulates at once
   // terms whose slice products stay within 2^24 whatever the slices are
   static constexpr int kDrain = ((1 << 24) - 512) / (2 * L << (2 * W - 2));
   // terms between two carries of the accumulators (their upper parts stay exact
@@ -862,9 +862,9 @@ __device__ __forceinline__ void columns(int d, int o, int nt, Terms a, bool rev,
 // parts takes its share of the column tiles.  The tiles are taken in groups of
 // consecutive ones (which share the Toeplitz fragments of their terms), dealt to the
 // warps of all parts longest first, back and forth, so that every warp has about the
-// same number of terms.  A correlation is run as a convolution with the series x reversed, and its result stored backwards.  Staging depth 2 claims the next job early
-// and copies its operands into a second buffer, if they are complete, while this one is
-// computed.
+// same number of terms.  A correlation is run as a convolution with the series x reversed,
+// and its result stored backwards.  Staging depth 2 claims the next job early and copies its
+// operands into a second buffer, if they are complete, while this one is computed.
 template <int K>
 __global__ void __launch_bounds__(mma_max_threads(K)) dag_mma_kernel(DagArgs a) {
   using M = Mma<K>;
@@ -959,8 +959,9 @@ __global__ void __launch_bounds__(mma_max_threads(K)) dag_mma_kernel(DagArgs a) 
         add_rows<K>(s1, s2, in.S, j, jb.kind == JOB_SUB ? -1 : 1, zrows);
     } else {
       const int32_t* my = reinterpret_cast<const int32_t*>(buf + lay.my);
-      const Found f = split_metas(reinterpret_cast<const int32_t*>(buf + lay.mx), reinterpret_cast<int32_t*>(buf + lay.ga),
-                                  d + 1, my, reinterpret_cast<int32_t*>(buf + lay.gb) + kPad, d + 1);
+      const Found f =
+          split_metas(reinterpret_cast<const int32_t*>(buf + lay.mx), reinterpret_cast<int32_t*>(buf + lay.ga), d + 1,
+                      my, reinterpret_cast<int32_t*>(buf + lay.gb) + kPad, d + 1);
       Terms at{};
       at.flat = is_flat<K>(f);
       at.gmax = at.flat ? f.gmax : 0;
@@ -1172,19 +1173,19 @@ void* mma_fn(bool tiled) {
 // Integer pipe's time over this form's, 7226 random polynomials (monomials of 2 to 16
 // variables), tenth percentile / median for uniform series; exponential ones with
 // coefficients of degree 0; coefficients falling by 2 bits a degree:
-//   k = 10, d 56-253, work 250-330 k   1.14 / 1.32   1.04 / 1.17   0.98 / 1.13
-//           d 254-471, 400-500 k       1.17 / 1.35   1.34 / 1.55   1.02 / 1.15
+//   k = 10, d 56-248, work 250-330 k   1.14 / 1.32   1.04 / 1.17   0.98 / 1.13
+//           d 249-471, 400-500 k       1.17 / 1.35   1.34 / 1.55   1.02 / 1.15
 //           tiles, 500-750 k           1.33 / 1.43   1.35 / 1.60   (zeros from d = 450 on)
-//   k = 8,  d 72-258, 330-400 k        1.12 / 1.23   0.99 / 1.10   0.94 / 1.07
-//           d 259-507, 750-1120 k      1.18 / 1.40   1.31 / 1.65   1.01 / 1.20
+//   k = 8,  d 72-252, 330-400 k        1.12 / 1.23   0.99 / 1.10   0.94 / 1.07
+//           d 253-513, 750-1120 k      1.18 / 1.40   1.31 / 1.65   1.01 / 1.20
 //           tiles, 1.75-3.25 M         1.05 / 1.25   1.41 / 1.85
 //   k = 4,  d 136-199, 640-800 k       1.10 / 1.16   1.03 / 1.08   0.93 / 1.04
-//           d 200-336, 1.2-1.8 M       1.19 / 1.33   1.25 / 1.47   1.00 / 1.13
-//           d 337-660, 2.8-5.2 M       1.25 / 1.32   1.45 / 1.80   0.98 / 1.14
+//           d 200-329, 1.2-1.8 M       1.19 / 1.33   1.25 / 1.47   1.00 / 1.13
+//           d 330-669, 2.8-5.2 M       1.25 / 1.32   1.45 / 1.80   0.98 / 1.14
 //           tiles, 640-800 k           1.05 / 1.10   1.77 / 2.20
-//   k = 5,  d 256-279, 1.2-1.8 M       1.18 / 1.37   1.40 / 1.46   1.04 / 1.16
-// and below the lines: k = 4, d 200-336, 400-640 k 0.88 / 0.98, d 337-660, 0.4-1.8 M 0.80 /
-// 0.97; k = 5, d 280-556 0.80 / 0.95, tiles 0.90 / 0.97; k = 8, d 259-507, 250-400 k 0.93 /
+//   k = 5,  d 256-277, 1.2-1.8 M       1.18 / 1.37   1.40 / 1.46   1.04 / 1.16
+// and below the lines: k = 4, d 200-329, 400-640 k 0.88 / 0.98, d 330-660, 0.4-1.8 M 0.80 /
+// 0.97; k = 5, d 278-556 0.80 / 0.95, tiles 0.90 / 0.97; k = 8, d 253-507, 250-400 k 0.93 /
 // 1.05, tiles of exponential series 0.71 / 0.78.
 bool mma_takes(int k, int d, const int32_t* supp_ptr, int32_t m0, int32_t m1, bool whole, size_t optin) {
   if (m0 >= m1 || !mma_has(k)) return false;
@@ -1224,7 +1225,8 @@ void* mma_kernel(int k, bool tiled) {
 
 size_t mma_smem_bytes(int k, int dmax, int depth) {
   const BufLayout lay = buf_layout(slice_digits(k), mma_stride(k), dmax + 1, dmax + 1);
-  return 4 * (static_cast<size_t>(kMiscWords) + static_cast<size_t>(depth >= 2 ? 2 : 1) * static_cast<size_t>(lay.words));
+  const size_t buffers = depth >= 2 ? 2 : 1;
+  return 4 * (kMiscWords + buffers * static_cast<size_t>(lay.words));
 }
 
 // Threads per CTA for degree dmax: as many warps as fill the registers with the CTAs that

@@ -116,8 +116,10 @@ bool whole_series_fits(int32_t k, int32_t arith, int32_t dmax, int32_t requested
 // The arithmetic of a plan: PES_ARITH_AUTO takes the integer arithmetic, on the tensor
 // cores where they are faster for every polynomial of it (one, or the P of a system with
 // first monomials poly_ptr).  The rule depends on the monomials' sizes, k and d alone, so
-// that every plan of a polynomial (whole series or tiles, alone, in a batch or without
-// allocations) holds its series in the same form and gives the same bits.
+// that every plan of a polynomial (whole series or tiles, alone or in a batch) holds its
+// series in the same form and gives the same bits; only where the series do not fit
+// (build_within_memory; the array of pes_eval_grad_static) does a call take the integer
+// pipe's shorter ones.
 int32_t resolve_arith(int32_t k, int32_t requested, int32_t d, const pes::Supports& sup,
                       const std::vector<int32_t>* poly_ptr, int optin) {
   if (requested != PES_ARITH_AUTO) return requested;
@@ -136,8 +138,9 @@ constexpr int32_t kStagedRows = 128;
 
 // Shared memory a CTA may take on this architecture (sm_103a).
 constexpr int kOptinBytes = 227 * 1024;
-static_assert(PES_ARITH_FP64 == pes::ARITH_FP64 && PES_ARITH_INT == pes::ARITH_INT && PES_ARITH_TENSOR == pes::ARITH_MMA,
-              "the arithmetics of the interface are the library's");
+static_assert(PES_ARITH_FP64 == pes::ARITH_FP64 && PES_ARITH_INT == pes::ARITH_INT &&
+                  PES_ARITH_TENSOR == pes::ARITH_MMA,
+              "the interface's arithmetics are the library's");
 
 int device_optin() {
   int dev = 0, optin = 0;
@@ -152,7 +155,6 @@ struct Exec {
   int32_t k = 0, arith = 0, threads = 128, ctas_per_sm = 0;
   int32_t smax = 0, dmax = 0;
   int32_t depth = 1, staging = 0;  // staging depth in use; requested (0 = automatic)
-  int32_t threads_req = 0;  // threads per CTA requested (0 = automatic)
   int32_t split = 1, split_req = 0;  // parts per convolution job in use; requested (0 = automatic)
   int32_t tile = 0;  // > 0: the tiled kernel, output tiles of this many coefficients (split = tiles per job)
   int32_t xrows = 0;  // tiled tensor-core kernel: coefficients of the first operand staged at once
@@ -280,7 +282,7 @@ struct Exec {
   pes_status init(int32_t k_, const pes_options& o, const std::vector<pes::InstInfo>& insts, size_t ws_words_) {
     k = k_;
     arith = o.arith;
-    threads = threads_req = o.threads;
+    threads = o.threads;
     ctas_per_sm = o.ctas_per_sm;
     timeout_ns = (o.timeout_ms > 0 ? o.timeout_ms : 60000) * 1000000LL;
     smax = 8;
@@ -324,9 +326,8 @@ struct Exec {
       if (arith == pes::ARITH_MMA && smem <= static_cast<size_t>(optin)) {
         // (tiles the integer pipe's kernel holds); a warp per group of column tiles
         // unless asked otherwise
-        threads = std::min(o.threads > 0 ? o.threads
-                                         : 32 * ((tile + 8 * pes::mma_group_tiles(k) - 1) / (8 * pes::mma_group_tiles(k))),
-                           pes::mma_max_threads(k));
+        constexpr int32_t group = 8 * pes::kMmaGroupTiles;
+        threads = std::min(o.threads > 0 ? o.threads : 32 * ((tile + group - 1) / group), pes::mma_max_threads(k));
         xrows = std::min(tile, kStagedRows);
         smem = pes::dag_tiled_smem_bytes(k, arith, tile, xrows);
       }
@@ -1582,7 +1583,8 @@ extern "C" pes_status pes_batch_check(pes_batch_t batch, void* stream) {
 extern "C" pes_status pes_auto_arith(const int32_t* supp_ptr, int32_t N, int32_t d, int32_t k, int32_t* arith) {
   if (!arith) return fail(PES_EINVAL, "arith is NULL");
   if (!valid_k(k)) return fail(PES_EUNSUPPORTED_K, "k must be one of 1,2,3,4,5,8,10");
-  if (N < 0 || d < 0 || d > pes::kMaxDegree || (N > 0 && !supp_ptr)) return fail(PES_EINVAL, "bad sizes or NULL pointer");
+  if (N < 0 || d < 0 || d > pes::kMaxDegree || (N > 0 && !supp_ptr))
+    return fail(PES_EINVAL, "bad sizes or NULL pointer");
   for (int32_t m = 0; m < N; ++m)
     if (supp_ptr[m + 1] <= supp_ptr[m]) return fail(PES_EINVAL, "empty monomial " + std::to_string(m));
   pes::Supports sup;

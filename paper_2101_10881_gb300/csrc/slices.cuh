@@ -102,7 +102,9 @@ PES_HD float meta_norm(int32_t q) {
 // 28-bit digits, L28 = digits_for_k(k, 28) of them.  Both see the same number: the
 // grid G of a sum whose largest contribution lies on grid g has B g - 28 G in
 // [B - 28, 16], and the bits of every contribution below the last 28-bit digit are
-// dropped (toward zero, digit by digit), in either form.
+// dropped (toward zero, digit by digit), in either form: less than one unit of that digit
+// a contribution, 2^-(53 k + 28) of the largest (a sum of 28-bit digits drops half a unit
+// of it; the products before drop less here than there).
 // ---------------------------------------------------------------------------
 template <int B>
 PES_HD int32_t sum_grid28(int32_t g) {

@@ -107,8 +107,9 @@ def test_systems_and_batches_have_the_bits_of_single_plans(torch, k):
     vo = go = 0
     for (supp, _, dd), c, z in zip(inst, cs, zs):
         pv, pg = pes.Plan(supp, n, dd, k, with_vjp=False, arith="tensor").eval_grad(cuda(torch, c), cuda(torch, z))
-        assert torch.equal(bv[vo:vo + pv.numel()], pv.reshape(-1)) and torch.equal(bg[go:go + pg.numel()], pg.reshape(-1))
-        vo, go = vo + pv.numel(), go + pg.numel()
+        nv, ng = pv.numel(), pg.numel()
+        assert torch.equal(bv[vo:vo + nv], pv.reshape(-1)) and torch.equal(bg[go:go + ng], pg.reshape(-1))
+        vo, go = vo + nv, go + ng
 
 
 def against_the_integer_pipe(torch, k, d, supp, n, coeff, inputs):
@@ -124,8 +125,8 @@ def against_the_integer_pipe(torch, k, d, supp, n, coeff, inputs):
     return infos
 
 
-@pytest.mark.parametrize("k,d,tile", [(8, 509, 0), (8, 520, 128), (5, 555, 0), (5, 600, 128), (4, 660, 0), (4, 700, 128),
-                                      (10, 471, 0), (10, 472, 128)])
+@pytest.mark.parametrize("k,d,tile", [(8, 513, 0), (8, 514, 128), (5, 563, 0), (5, 564, 128), (4, 669, 0),
+                                      (4, 670, 128), (10, 471, 0), (10, 472, 128)])
 def test_whole_series_and_tiles(torch, k, d, tile):
     """The tiled kernel takes the degrees whose staged pairs do not fit in shared memory, also
     where 28-bit digits would."""
@@ -167,3 +168,25 @@ def test_products_far_below_the_smallest_double(torch, k):
     assert got[0][0][0, 0] == 1.0
     for a, b in zip(*got):
         assert normwise_err(a, b) <= close(k)
+
+
+@pytest.mark.parametrize("k", KT)
+def test_one_product_is_exact_to_the_last_limb(torch, k):
+    """One product of two series against rationals: what the tensor form drops of a product and
+    the rounding to k limbs together stay below 2^-(53 k - 2) of the sum of the terms'
+    magnitudes (2^-(53 k) from the rounding, less than 2^-(53 k) dropped)."""
+    from fractions import Fraction
+    from tests.exact import series_fractions
+    rng = np.random.default_rng(k)
+    d = 40
+    inputs = random_md(rng, k, (2, d + 1))
+    coeff = np.zeros((k, 2, d + 1))
+    coeff[0, 1, 0] = 1.0
+    plan = pes.Plan([[0, 1]], 2, d, k, with_vjp=False, arith="tensor")
+    v, _ = plan.eval_grad(cuda(torch, coeff), cuda(torch, inputs))
+    plan.check()
+    got = series_fractions(v.cpu().numpy())
+    x, y = series_fractions(inputs)
+    for j in range(d + 1):
+        terms = [x[i] * y[j - i] for i in range(j + 1)]
+        assert abs(got[j] - sum(terms)) <= sum(abs(t) for t in terms) * Fraction(1, 2 ** (53 * k - 2))
