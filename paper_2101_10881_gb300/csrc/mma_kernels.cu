@@ -281,9 +281,11 @@ __device__ __forceinline__ void nonzero_terms(const volatile Range* r, int jlo, 
 }
 
 // The terms [x0, x1) that meet nonzero coefficients in the columns [c0, terms) of an
-// output tile (into the Range of the misc words), by the whole CTA.  (Not inlined: the
-// kernel around it has no register to spare.)
-__device__ __noinline__ void tile_range(const int32_t* gx, const int32_t* gy, int step, int terms, int c0) {
+// output tile (into the Range of the misc words), by the whole CTA.  `either`: either
+// operand may be the Toeplitz one; true if it is better the second, which has fewer.  (Not
+// inlined: the kernel around it has no register to spare.)
+__device__ __noinline__ bool tile_range(const int32_t* gx, const int32_t* gy, int step, int terms, int c0,
+                                        bool either) {
   Range* r = reinterpret_cast<Range*>(sm + kRangeWord);
   if (threadIdx.x == 0) *r = Range{terms, 0, terms, 0, 0};
   __syncthreads();
@@ -306,12 +308,15 @@ __device__ __noinline__ void tile_range(const int32_t* gx, const int32_t* gy, in
     atomicMax(&r->y1, y1);
   }
   __syncthreads();
+  x0 = r->x0, x1 = r->x1, y0 = r->y0, y1 = r->y1;
+  const bool swap = either && y1 - y0 < x1 - x0;
+  __syncthreads();
   if (threadIdx.x == 0) {
-    const int begin = max(r->x0, c0 - r->y1 + 1), end = min(r->x1, terms - r->y0);
-    r->x0 = begin;
-    r->x1 = end;
+    r->x0 = max(swap ? y0 : x0, c0 - (swap ? x1 : y1) + 1);
+    r->x1 = min(swap ? y1 : x1, terms - (swap ? x0 : y0));
   }
   __syncthreads();
+  return swap;
 }
 
 // The columns' grids lie close enough for their rows to be shifted to the largest.
@@ -1070,20 +1075,23 @@ __global__ void __launch_bounds__(mma_max_threads(K)) dag_mma_tiled_kernel(DagAr
         // columns [c0, c0 + jn); of a correlation, those of the reversed result, whose
         // column operand is the reversed first series
         const int c0 = conv ? tile * D : d + 1 - tile * D - jn;
-        const int32_t* xs = conv ? s1 : s2;  // the Toeplitz operand
-        const int32_t* ys = conv ? s2 : s1;
-        const int32_t* gX = xs + static_cast<long long>(S) * L;
-        const int32_t* gY = ys + static_cast<long long>(S) * L;
         const int terms = c0 + jn;  // of the tile's longest coefficient
+        // Only chunks of terms that meet nonzero coefficients in a column of the tile are
+        // staged, and the operand with fewer of them is the Toeplitz one (inputs of degree 1;
+        // integer pipe, all chunks, here: 8 products of 16, d = 1023, k = 10: 3.1, 8.8,
+        // 2.0 ms; 40 products of 4, d = 600, k = 10: 0.74, 1.53, 0.69 ms).
+        volatile Range* range = reinterpret_cast<volatile Range*>(sm + kRangeWord);
+        const long long metas = static_cast<long long>(S) * L;
+        const bool first = tile_range((conv ? s1 : s2) + metas, conv ? s2 + metas : s1 + metas + d, conv ? 1 : -1,
+                                      terms, c0, conv) != conv;
+        const int32_t* xs = first ? s1 : s2;  // the Toeplitz operand
+        const int32_t* ys = first ? s2 : s1;
+        const int32_t* gX = xs + metas;
+        const int32_t* gY = ys + metas;
         const int ntiles = (jn + 7) / 8;
         // groups of consecutive column tiles, longest first, in passes of one per warp
         const int gsz = min(NT, (ntiles + warps - 1) / warps);
         const int ngroups = (ntiles + gsz - 1) / gsz;
-        // Only chunks of terms that meet nonzero coefficients in a column of the tile are staged
-        // (8 products of 16, d = 1023, k = 10, inputs of degree 1: integer pipe 3.1 ms, all
-        // chunks 8.8 ms, here 2.8 ms).
-        volatile Range* range = reinterpret_cast<volatile Range*>(sm + kRangeWord);
-        tile_range(gX, conv ? gY : gY + d, conv ? 1 : -1, terms, c0);
         for (int p0 = 0; p0 < ngroups; p0 += warps) {
           Group<K> grp;
           const int o = (p0 + warp) * gsz;
