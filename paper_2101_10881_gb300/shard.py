@@ -32,8 +32,10 @@ class ShardPlan:
         self.supports = [list(s) for s in supports[self.m_begin:self.m_end]]
         ex = None if exponents is None else [list(e) for e in exponents[self.m_begin:self.m_end]]
         self.n, self.d, self.k = int(n), int(d), int(k)
-        # the automatic arithmetic goes by a plan's monomials: here by the whole polynomial's
-        if opts.get("arith", "auto") in ("auto", pes.ARITH["auto"]):
+        # The automatic arithmetic goes by a plan's monomials: here by the whole polynomial's.
+        # (Several ranks cannot fall back each for itself where a share's tensor-core series,
+        # up to 1.54 times as long, exceed the device memory: arith="int" on all of them does.)
+        if self.world > 1 and opts.get("arith", "auto") in ("auto", pes.ARITH["auto"]):
             opts["arith"] = pes.auto_arith(supports, d, k)
         self.plan = pes.Plan(self.supports, n, d, k, exponents=ex, with_vjp=False, **opts)
 
