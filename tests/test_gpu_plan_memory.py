@@ -1,10 +1,11 @@
-"""A plan or batch whose series fit the device memory as 28-bit digits only is built for the
+"""A plan, batch or single rank whose series fit the device memory as 28-bit digits only is built for the
 integer pipe, where the automatic arithmetic would take the longer series of the tensor cores."""
 import itertools
 
 import pytest
 
 from paper_2101_10881_gb300 import pes
+from paper_2101_10881_gb300.shard import ShardPlan
 
 pytestmark = pytest.mark.gpu
 
@@ -17,8 +18,9 @@ def torch():
     return _t
 
 
-@pytest.mark.parametrize("batch", [False, True])
-def test_falls_back_to_the_integer_pipe(torch, batch):
+@pytest.mark.parametrize("kind", ["plan", "batch", "rank"])
+def test_falls_back_to_the_integer_pipe(torch, kind):
+    batch = kind == "batch"
     k, d, n = 5, 270, 200
     supp = [list(s) for s in itertools.combinations(range(n), 2)]
     gen = torch.Generator(device="cuda")
@@ -32,6 +34,8 @@ def test_falls_back_to_the_integer_pipe(torch, batch):
     def build(arith):
         if batch:
             return pes.Batch([(supp, n, d)], k, arith=arith)
+        if kind == "rank":
+            return ShardPlan(supp, n, d, k, 1, 0, arith=arith).plan
         return pes.Plan(supp, n, d, k, with_vjp=False, arith=arith)
 
     v, g = (torch.empty((k, rows, d + 1), dtype=torch.float64, device="cuda") for rows in (1, n))
