@@ -1473,6 +1473,14 @@ __device__ __forceinline__ void add_round(const AddArgs& a, long long w, const l
   from_digits<K, NW, B>(E, gmax + 1, dst, ao.dst_lstride);
 }
 
+// CTAs per SM that the registers of the addition kernels for tables of few, long sums are
+// planned for (0: the compiler's choice).  Left to itself the compiler takes 80 registers
+// at k = 8, and the loads of a lane's contributions follow one another: sums of 4414 and
+// 441 products, d = 6, 65 us instead of 47.  (In the kernels of larger tables, whose
+// warps hide one another's loads, the bound costs 1 to 3 %, and at the tensor cores' rows,
+// which are summed in half the registers, 2 %.)
+__host__ __device__ constexpr int add_min_ctas(int arith) { return arith == ARITH_MMA ? 0 : 2; }
+
 // An output coefficient is summed by a.group_warps warps (GROUPED; block barriers combine
 // them) or one.  A block sums a.rounds times as many as it has groups, one after another,
 // and keeps the sums in shared memory; then it rounds all of them at once, one per lane.
@@ -1543,7 +1551,7 @@ void round_sums_host_k(const RoundArgs& a) {
 }
 
 template <int K, int AR>
-__global__ void __launch_bounds__(256) add_kernel_grouped(AddArgs a, long long items) {
+__global__ void __launch_bounds__(256, add_min_ctas(AR)) add_kernel_grouped(AddArgs a, long long items) {
   add_body<K, AR, true>(a, items, blockIdx.x);
 }
 
@@ -1569,7 +1577,7 @@ __global__ void __launch_bounds__(256) add_kernel_pair(AddArgs a0, long long ite
 }
 
 template <int K, int AR>
-__global__ void __launch_bounds__(256) add_kernel_pair_grouped(AddArgs a0, long long items0, AddArgs a1,
+__global__ void __launch_bounds__(256, add_min_ctas(AR)) add_kernel_pair_grouped(AddArgs a0, long long items0, AddArgs a1,
                                                                long long items1, unsigned nb0) {
   add_pair_body<K, AR, true>(a0, items0, a1, items1, nb0);
 }
