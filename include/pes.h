@@ -92,8 +92,8 @@ typedef struct {
                           are tried when autotuning) */
   int32_t split;       /* parts per convolution job (integer pipe, tensor cores): 1, 2, 4, 8 or 16; each
                           part computes the output coefficients of a contiguous range of coefficient
-                          pairs (j, d-j), so a job's dependants wait for all its parts; more parts shorten the chains of long
-                          monomials; 0 = automatic: the parts double while the table's average layer, times
+                          pairs (j, d-j), so a job's dependants wait for all its parts; more parts
+                          shorten the chains of long monomials; 0 = automatic: the parts double while the table's average layer, times
                           the parts, holds fewer jobs than the launch has CTAs and every part keeps at
                           least 8 coefficient pairs (the p2-like workload at d=152, k=10: 1 for its 128
                           monomials, 2 for 64 of them, 4 for 32, 8 for 16 or fewer; p3: 1; tensor cores:

@@ -22,7 +22,7 @@
 //   so every lane shifts its own column by an address;
 // - blocks above the diagonal (rows whose slices all lie above the column slices)
 //   are zero and not issued.
-// tcgen05 has four times the rate, but needs the Toeplitz matrix in shared memory
+// tcgen05 has three times the rate, but needs the Toeplitz matrix in shared memory
 // (one copy of x per row of a core matrix) and 128 rows for every k; reading that
 // operand (32 cycles a step against 16 to 40 for the columns here) would bound it at
 // about the time of this form.
