@@ -87,3 +87,23 @@ def test_short_series_take_less_time(torch, k, d, n, parts):
             b.synchronize()
             best[name] = min(best.get(name, 1e9), a.elapsed_time(b))
     assert best["short"] < (0.75 if parts == "both" else 0.5) * best["full"], best
+
+
+@pytest.mark.parametrize("pattern", PATTERNS)
+@pytest.mark.parametrize("k,d,n", [(10, 95, 8), (4, 152, 8), (8, 101, 8), (5, 67, 8)])
+def test_tiles_have_the_bits_of_whole_series(torch, k, d, n, pattern):
+    """The tiled kernel exchanges a product's operands by where their zeros lie and stages fewer
+    chunks; whole series clip their terms: the same sums."""
+    rng = np.random.default_rng(d)
+    supp = [list(s) for m in (2, 3) for s in itertools.combinations(range(n), m)]
+    coeff, inputs = PATTERNS[pattern](random_md(rng, k, (len(supp) + 1, d + 1)), random_md(rng, k, (n, d + 1)))
+    C, Z, U = (torch.from_numpy(np.ascontiguousarray(a)).cuda() for a in (coeff, inputs, random_md(rng, k, (d + 1,))))
+    U[:, 5:] = 0
+    got = []
+    for opts in ({}, {"tile": 16}, {"tile": 48}, {"split": 2, "staging": 2}):
+        plan = pes.Plan(supp, n, d, k, arith="tensor", **opts)
+        got.append([*plan.eval_grad(C, Z), *plan.vjp(C, Z, U, reuse_forward=True)])
+        plan.check()
+    for other in got[1:]:
+        for a, b in zip(got[0], other):
+            assert torch.equal(a, b)
